@@ -117,6 +117,9 @@ cwt_status run_execute(cwt_plan_s *p, const void *sig, void *oc, void *op, void 
 
 void free_plan_memory(cwt_plan_s *p) {
     cwtk::free_batch_state(p->batch);
+    cwtk::free_zoom_plan(p->zoom);
+    p->zoom = nullptr;
+    cudaFree(p->rest_list);
     p->batch = nullptr;
     cudaFree(p->bank);
     cudaFree(p->band);
@@ -353,6 +356,7 @@ cwt_status cwt_plan_create(cwt_plan *out, int channels, int samples, double fs,
         }
     }
     if (e == cudaSuccess) e = cwtk::launch_bank(p, st);
+    if (e == cudaSuccess) e = cwtk::zoom_plan_create(p, st);
     if (e == cudaSuccess && tc) {
         e = cwtk::dmalloc(&p->tc_chmax, sizeof(float) * (size_t)channels);
         if (e == cudaSuccess) e = cwtk::dmalloc(&p->tc_wl1, sizeof(float) * (size_t)n_freqs);

@@ -27,6 +27,7 @@ template <int N, typename IO>
 __global__ void __cluster_dims__(N / kClPoints, 1, 1) __launch_bounds__(kClThreads, 1)
 cl_forward_kernel(const IO *__restrict__ x, int n, float2 *__restrict__ spec,
                   const float2 *__restrict__ tw) {
+    griddep_launch();
     extern __shared__ float2 clsm[];
     constexpr int CL = ClusterShape<N>::CL;
     const int row = blockIdx.x / CL;
@@ -58,7 +59,8 @@ struct ClArgs {
     const int *band;
     const float2 *tw;
     void *out_c, *out_p, *out_ph;
-    int S, n_out, sub;
+    const int *list;  // [ns] the scales to run, or NULL: all (ns = S)
+    int S, ns, n_out, sub;
 };
 
 // PLAIN: no decimation (output o = t), so each output needs only the crop
@@ -67,10 +69,13 @@ template <int N, typename IO, bool PLAIN>
 __global__ void __cluster_dims__(N / kClPoints, 1, 1) __launch_bounds__(kClThreads, 1)
 cl_scale_block_kernel(const ClArgs a) {
     using V2 = typename IO2c<IO>::type;
+    griddep_launch();
     extern __shared__ float2 clsm[];
     constexpr int CL = ClusterShape<N>::CL;
     const int row = blockIdx.x / CL;
-    const int c = row / a.S, s = row - c * a.S;
+    const int c = row / a.ns;
+    int s = row - c * a.ns;
+    if (a.list) s = a.list[s];
     const float2 *X = a.spec + (size_t)c * N;
     const float *W = a.bank + (size_t)s * N;
     const int b0 = a.band[2 * s], B = a.band[2 * s + 1];
@@ -82,7 +87,7 @@ cl_scale_block_kernel(const ClArgs a) {
         }
         return make_float2(0.f, 0.f);
     };
-    const size_t obase = (size_t)row * (size_t)a.n_out;
+    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
     V2 *oc = (V2 *)a.out_c;
     IO *op = (IO *)a.out_p;
     IO *oph = (IO *)a.out_ph;
@@ -212,9 +217,11 @@ cudaError_t launch_scale_block_cluster(const cwt_plan_s *p, void *out_c, void *o
     a.out_p = out_p;
     a.out_ph = out_ph;
     a.S = p->S;
+    a.ns = p->rest_scales;
+    a.list = p->rest_list;
     a.n_out = p->n_out;
     a.sub = p->d;  // fold is 1 on this path
-    const int rows = p->C * p->S;
+    const int rows = p->C * a.ns;
     const int log2n = ilog2c(p->N);
     if (p->io == CWT_DTYPE_F64) return cl_sb_dispatch<double>(log2n, a, rows, st);
     return cl_sb_dispatch<float>(log2n, a, rows, st);

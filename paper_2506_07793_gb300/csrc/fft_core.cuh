@@ -60,6 +60,13 @@ __host__ __device__ constexpr float cos32(int m) {
 }
 __host__ __device__ constexpr float sin32(int m) { return cos32(m + 24); }
 
+// Programmatic dependent launch (griddepcontrol, sm_90 and up): let the next
+// kernel of the stream start once every CTA of this one has got here; wait
+// until the kernels before this one have completed and their writes are
+// visible.  Without the launch attribute on the next kernel both do nothing.
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Complex add / subtract as one packed FP32x2 instruction (add/sub.rn.f32x2,
 // sm_100 and later): the same round-to-nearest result per component as two
 // scalar adds, in half the issue slots.  (A packed multiply-add form of cmul

@@ -20,6 +20,7 @@ template <int N, typename IO>
 __global__ void __launch_bounds__(RowConfig<N>::THREADS)
 forward_kernel(const IO *__restrict__ x, int C, int n, float2 *__restrict__ spec,
                const float2 *__restrict__ tw) {
+    griddep_launch();
     using RC = RowConfig<N>;
     extern __shared__ float2 smem2[];
     const int rl = threadIdx.x / RC::T, j = threadIdx.x % RC::T;

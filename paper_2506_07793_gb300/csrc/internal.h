@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "cwt.h"
+#include "fft_core.cuh"
 #include "mixed_radix.cuh"
 
 namespace cwtk {
@@ -45,8 +46,14 @@ cudaError_t hmalloc(T **p, size_t bytes) {
 // ordinary build.
 bool check_collect(std::string *where);
 
-// Per-device FP32 twiddle table exp(2 pi i m / 2^17), built in FP64 on first use.
+// Per-device FP32 twiddle table exp(2 pi i m / 2^17), built in FP64 on first
+// use, and behind it the tables of 2^16, 2^15, ... 2 points (twiddles_pow2).
 cudaError_t device_twiddles(const float2 **out);
+// The table of L = 2^l points, l <= 17, given device_twiddles' pointer.
+inline const float2 *twiddles_pow2(const float2 *tw, int L) { return tw + 2 * kTwN - 2 * L; }
+
+struct ZoomPlan;  // zoom.cu
+void free_zoom_plan(ZoomPlan *z);
 
 struct BatchState;
 void free_batch_state(BatchState *b);
@@ -92,6 +99,9 @@ struct cwt_plan_s {
     float *tc_chmax = nullptr;  // tensor-core plans: [C] max |Re|, |Im| of each spectrum
     float *tc_wl1 = nullptr;    // tensor-core plans: [S] sum of |W_s| over the band
     const float2 *tw = nullptr;
+    cwtk::ZoomPlan *zoom = nullptr;   // scales run by output residue classes (zoom.cu), or null
+    int rest_scales = 0;              // the other scales: how many, and which (null: all S)
+    int *rest_list = nullptr;
     size_t bytes = 0;
     double bank_ms = 0;
 
@@ -195,6 +205,13 @@ cudaError_t launch_scale_block(const cwt_plan_s *p, void *out_c, void *out_p, vo
                                cudaStream_t st);
 cudaError_t launch_fft(const float2 *in, float2 *out, int log2n, int batch, int sign,
                        const float2 *tw, cudaStream_t st);
+// Narrow-band scales by output residue classes (zoom.cu).  zoom_plan_create
+// picks each scale's transform from its band (the bank is in place), sets
+// p->zoom, p->rest_scales and p->rest_list, and leaves p->zoom null when no
+// scale takes it.
+cudaError_t zoom_plan_create(cwt_plan_s *p, cudaStream_t st);
+cudaError_t launch_scale_block_zoom(const cwt_plan_s *p, float2 *out_c, float *out_p, float *out_ph,
+                                    cudaStream_t st);
 // Tensor-core inverse FFTs (tc_scale_block.cu): per-channel spectrum bounds
 // after the forward FFT, per-scale band sums at plan creation, the scale block.
 cudaError_t launch_tc_row_bounds(const cwt_plan_s *p, cudaStream_t st);
@@ -207,9 +224,8 @@ cudaError_t launch_scale_block_cluster(const cwt_plan_s *p, void *out_c, void *o
                                        cudaStream_t st);
 cudaError_t launch_fft_cluster(const float2 *in, float2 *out, int log2n, int batch, int sign,
                                const float2 *tw, cudaStream_t st);
-// prepare_only: build the work items, generate missing banks and autotune a
-// new batch shape (its candidate runs write valid outputs); otherwise launch
-// the chosen schedule's graph once.
+// prepare_only: generate missing banks and build the work items of a new batch
+// shape; otherwise launch what the last such call prepared.
 // Smooth lengths (smooth.cu): schedule, per-N twiddles, kernels.
 bool mr_schedule(int N, MrSchedule *out);
 cudaError_t make_twiddles_n(int N, float2 *tw, cudaStream_t st);

@@ -409,7 +409,7 @@ cudaError_t jit_cl_sb_launch(const cwt_plan_s *p, const ClMrArgs &a, cudaStream_
     ClMrArgs args = a;
     MrSchedule sch = p->sch;
     void *params[] = {&args, &sch};
-    const unsigned grid = (unsigned)(p->C * p->S * k->cl);
+    const unsigned grid = (unsigned)(p->C * a.ns * k->cl);
     const CUresult r = driver().launch_kernel(k->sb, grid, 1, 1, (unsigned)k->threads, 1, 1, (unsigned)k->smem,
                                               (CUstream)st, params, nullptr);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
@@ -482,7 +482,8 @@ JitKernels *jit_tune(cwt_plan_s *p, cudaStream_t st, std::string *log) {
     a.out_c = oc;
     a.out_p = op;
     a.out_ph = oph;
-    a.S = p->S;
+    a.list = nullptr;
+    a.S = a.ns = p->S;
     a.n_out = p->n_out;
     a.sub = p->d;
     a.total_rows = trows;
@@ -496,7 +497,8 @@ JitKernels *jit_tune(cwt_plan_s *p, cudaStream_t st, std::string *log) {
     ca.out_c = oc;
     ca.out_p = op;
     ca.out_ph = oph;
-    ca.S = p->S;
+    ca.list = nullptr;
+    ca.S = ca.ns = p->S;
     ca.n_out = p->n_out;
     ca.sub = p->d;
     ca.f64 = p->io == CWT_DTYPE_F64;

@@ -30,7 +30,8 @@ struct SBArgs {
     const int *band;     // [S][2]
     const float2 *tw;
     void *out_c, *out_p, *out_ph;
-    int C, S, N, n_out, fold, sub, rows;
+    const int *list;     // [ns] the scales to run, or NULL: all (ns = S)
+    int C, S, ns, N, n_out, fold, sub, rows;
 };
 
 template <typename IO> struct IO2;
@@ -49,11 +50,13 @@ scale_block_kernel(const SBArgs a) {
     using RC = RowConfig<M>;
     using V2 = typename IO2<IO>::type;
     extern __shared__ float2 smem2[];
+    griddep_launch();
     const int rl = threadIdx.x / RC::T, j = threadIdx.x % RC::T;
     const int row = blockIdx.x * RC::ROWS + rl;
     const bool act = row < a.rows;
-    const int c = act ? row / a.S : 0;
-    const int s = act ? row - c * a.S : 0;
+    const int c = act ? row / a.ns : 0;
+    int s = act ? row - c * a.ns : 0;
+    if (a.list) s = a.list[s];
     float2 *sm = smem2 + rl * FftShape<M, RC::R>::SMEM_F2;
 
     const float2 *X = a.spec + (size_t)c * (size_t)a.N;
@@ -98,7 +101,7 @@ scale_block_kernel(const SBArgs a) {
         return acc;
     };
 
-    const size_t obase = (size_t)row * (size_t)a.n_out;
+    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
     V2 *oc = (V2 *)a.out_c;
     IO *op = (IO *)a.out_p;
     IO *oph = (IO *)a.out_ph;
@@ -173,8 +176,8 @@ cudaError_t sb_dispatch(int log2m, const SBArgs &a, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_scale_block(const cwt_plan_s *p, void *out_c, void *out_p, void *out_ph,
-                               cudaStream_t st) {
+// The whole-row kernels over the scales of p->rest_list.
+static cudaError_t launch_whole_rows(const cwt_plan_s *p, void *out_c, void *out_p, void *out_ph, cudaStream_t st) {
     if (p->mr) return launch_scale_block_mr(p, out_c, out_p, out_ph, st);
     if (p->M > kMaxFft) return launch_scale_block_cluster(p, out_c, out_p, out_ph, st);
     SBArgs a;
@@ -187,14 +190,27 @@ cudaError_t launch_scale_block(const cwt_plan_s *p, void *out_c, void *out_p, vo
     a.out_ph = out_ph;
     a.C = p->C;
     a.S = p->S;
+    a.ns = p->rest_scales;
+    a.list = p->rest_list;
     a.N = p->N;
     a.n_out = p->n_out;
     a.fold = p->fold;
     a.sub = p->sub;
-    a.rows = p->C * p->S;
+    a.rows = p->C * a.ns;
     const int log2m = ilog2c(p->M);
     if (p->io == CWT_DTYPE_F64) return sb_dispatch<double>(log2m, a, st);
     return sb_dispatch<float>(log2m, a, st);
 }
 
+cudaError_t launch_scale_block(const cwt_plan_s *p, void *out_c, void *out_p, void *out_ph,
+                               cudaStream_t st) {
+    // scales whose band is narrow run by residue classes, the rest as whole rows
+    if (p->rest_scales > 0) {
+        const cudaError_t e = launch_whole_rows(p, out_c, out_p, out_ph, st);
+        if (e != cudaSuccess) return e;
+    }
+    return p->zoom ? launch_scale_block_zoom(p, (float2 *)out_c, (float *)out_p, (float *)out_ph, st) : cudaSuccess;
+}
+
 }  // namespace cwtk
+

@@ -347,9 +347,11 @@ cudaError_t launch_scale_block_mr(const cwt_plan_s *p, void *out_c, void *out_p,
     a.out_p = out_p;
     a.out_ph = out_ph;
     a.S = p->S;
+    a.ns = p->rest_scales;
+    a.list = p->rest_list;
     a.n_out = p->n_out;
     a.sub = p->d;
-    a.total_rows = p->C * p->S;
+    a.total_rows = p->C * a.ns;
     a.f64 = p->io == CWT_DTYPE_F64;
     if (p->jit) return jit_sb_launch(p, a, st);
     if (p->sch.fixed >= 0) return mr_fixed_sb_launch(p, a, st);

@@ -30,6 +30,8 @@ cudaError_t launch_scale_block_mr_cluster(const cwt_plan_s *p, void *out_c, void
     a.out_p = out_p;
     a.out_ph = out_ph;
     a.S = p->S;
+    a.ns = p->rest_scales;
+    a.list = p->rest_list;
     a.n_out = p->n_out;
     a.sub = p->d;
     a.f64 = p->io == CWT_DTYPE_F64;

@@ -18,7 +18,8 @@ struct ClMrArgs {
     const float2 *twL;   // exp(2 pi i m / NL), m < NL: the local passes
     const float2 *twN;   // exp(2 pi i m / N), m < N: the cross-CTA stage
     void *out_c, *out_p, *out_ph;
-    int S, n_out, sub, f64;
+    const int *list;  // [ns] the scales to run, or null: all (ns = S)
+    int S, ns, n_out, sub, f64;
 };
 
 namespace cl_mr {
@@ -153,12 +154,15 @@ __device__ __forceinline__ void cross(const float2 *sm, const float2 *__restrict
 template <int CL, class FX>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(max_threads<FX>(), min_blocks<FX>())
 scale_block_kernel(const ClMrArgs a, const MrSchedule sch) {
+    griddep_launch();
     extern __shared__ float2 mrsm[];
     float2 *sm = mrsm;
     const int NL = local_n<FX>(sch), N = CL * NL;
     const int rank = (int)cluster_rank();
     const int row = (int)blockIdx.x / CL;
-    const int c = row / a.S, s = row - c * a.S;
+    const int c = row / a.ns;
+    int s = row - c * a.ns;
+    if (a.list) s = a.list[s];
     const float2 *X = a.spec + (size_t)c * N;
     const float *W = a.bank + (size_t)s * N;
     const int b0 = a.band[2 * s], B = a.band[2 * s + 1];
@@ -170,7 +174,7 @@ scale_block_kernel(const ClMrArgs a, const MrSchedule sch) {
     const BandFirst first_nz{X, W, m_first, Bm, NL, rank, CL};
     local_row<FX, +1>(sch, sm, a.twL, (int)threadIdx.x, Bm <= NL / first_radix<FX>(sch), load, first_nz);
     cluster_sync();  // every CTA's A_c in natural order
-    const size_t obase = (size_t)row * (size_t)a.n_out;
+    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
     const int sub = a.sub, n_out = a.n_out;
     auto out = [&](int t, float2 v) {
         int o = t;
@@ -197,6 +201,7 @@ template <int CL, class FX>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(max_threads<FX>(), min_blocks<FX>())
 forward_kernel(const void *__restrict__ x, int f64, int n, float2 *__restrict__ spec,
                const float2 *__restrict__ twL, const float2 *__restrict__ twN, const MrSchedule sch) {
+    griddep_launch();
     extern __shared__ float2 mrsm[];
     float2 *sm = mrsm;
     const int NL = local_n<FX>(sch), N = CL * NL;

@@ -18,7 +18,8 @@ struct MrArgs {
     const int *band;
     const float2 *twN;
     void *out_c, *out_p, *out_ph;
-    int S, n_out, sub, total_rows, f64;
+    const int *list;  // [ns] the scales to run, or null: all (ns = S)
+    int S, ns, n_out, sub, total_rows, f64;
 };
 
 __device__ __noinline__ inline void mr_phase_f(float *dst, float2 v) { *dst = phase_atan2(v.y, v.x); }
@@ -32,11 +33,14 @@ __device__ __noinline__ inline void mr_phase_d(double *dst, float2 v) { *dst = (
 template <bool LIN, typename RunRow>
 __device__ __forceinline__ void mr_sb_row(const MrArgs &a, int N, int T, int R0, const RowSlot &rs, int rows,
                                           const RunRow &run_row) {
+    griddep_launch();
     extern __shared__ float2 mrsm[];
     const int row = rs.active ? (int)blockIdx.x * rows + rs.rr : 0;
     const int rr = rs.rr < rows ? rs.rr : 0;
     float2 *sm = mrsm + (size_t)rr * (N + (N >> 4));
-    const int c = row / a.S, s = row - c * a.S;
+    const int c = row / a.ns;
+    int s = row - c * a.ns;
+    if (a.list) s = a.list[s];
     const float2 *X = a.spec + (size_t)c * N;
     const float *W = a.bank + (size_t)s * N;
     const int b0 = a.band[2 * s], B = a.band[2 * s + 1];
@@ -68,7 +72,7 @@ __device__ __forceinline__ void mr_sb_row(const MrArgs &a, int N, int T, int R0,
     if (!rs.active) return;
     // epilogue: crop to t < n, keep t = sub * o, write the requested outputs
     // (consecutive threads take consecutive o: coalesced stores)
-    const size_t obase = (size_t)row * (size_t)a.n_out;
+    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
     const int sub = a.sub, n_out = a.n_out;
     if (a.f64) {
         double2 *oc = (double2 *)a.out_c + obase;
@@ -127,6 +131,7 @@ template <class FX>
 __global__ void __launch_bounds__(FX::THREADS, FX::MINB)
 mr_fixed_forward_kernel(const void *__restrict__ x, int f64, int n, float2 *__restrict__ spec,
                         const float2 *__restrict__ twN, int C) {
+    griddep_launch();
     extern __shared__ float2 mrsm[];
     constexpr int N = FX::N;
     RowSlot rs;

@@ -52,6 +52,7 @@ template <int RA, int RB>
 __global__ void __launch_bounds__(kMrThreads, 1)
 mr_forward_kernel(const void *__restrict__ x, int f64, int n, float2 *__restrict__ spec,
                   const float2 *__restrict__ twN, const MrSchedule sch, int rows, int C) {
+    griddep_launch();
     extern __shared__ float2 mrsm[];
     const int N = sch.N;
     const RowSlot rs = row_slot(sch, rows, C);

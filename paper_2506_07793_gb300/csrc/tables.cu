@@ -42,12 +42,18 @@ namespace cwtk {
 
 namespace {
 
+// The tables of 2^17, 2^16, ... 2 points one after the other (twiddles_pow2).
 __global__ void twiddle_kernel(float2 *tw) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < kTwN) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int L = kTwN, m = i;
+    while (L > 2 && m >= L) {
+        m -= L;
+        L >>= 1;
+    }
+    if (m < L) {
         double s, c;
-        sincospi(2.0 * (double)m / (double)kTwN, &s, &c);
-        tw[m] = make_float2((float)c, (float)s);
+        sincospi(2.0 * (double)m / (double)L, &s, &c);
+        tw[i] = make_float2((float)c, (float)s);
     }
 }
 
@@ -190,7 +196,7 @@ cudaError_t device_twiddles(const float2 **out) {
     std::lock_guard<std::mutex> lk(g_tw_mutex);
     if (!g_tw[dev]) {
         float2 *tw = nullptr;
-        e = cwtk::dmalloc(&tw, sizeof(float2) * kTwN);
+        e = cwtk::dmalloc(&tw, sizeof(float2) * 2 * kTwN);
         if (e != cudaSuccess) return e;
         cudaStream_t st;
         e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
@@ -198,7 +204,7 @@ cudaError_t device_twiddles(const float2 **out) {
             cudaFree(tw);
             return e;
         }
-        twiddle_kernel<<<kTwN / 256, 256, 0, st>>>(tw);
+        twiddle_kernel<<<2 * kTwN / 256, 256, 0, st>>>(tw);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaStreamDestroy(st);

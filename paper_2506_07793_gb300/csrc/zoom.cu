@@ -1,0 +1,409 @@
+// zoom.cu -- which scales run by output residue classes (zoom.cuh), with which
+// transform, and their launches.
+//
+// A row of N bins decimated by d is evaluated on the M = N / gcd(N, d) points
+// that contain every kept sample (the spectral fold is implied: bins are
+// taken mod M).  A scale whose band has B bins can run any instance with
+// Q >= B and Q a divisor of M; the choice depends on the length and the bands
+// alone, so that a shard of the channels gives the same bits as the whole.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <new>
+#include <numeric>
+#include <vector>
+
+#include "internal.h"
+#include "zoom.h"
+
+namespace cwtk {
+
+namespace {
+
+struct ZoomInst {
+    int QA, Q, NB, P, T, LAST;
+    float cost;  // ps per point
+};
+
+// instance i of zoom_list.h (the groups list them out of order)
+const ZoomInst &inst(int i) {
+    static const std::vector<ZoomInst> table = [] {
+        std::vector<ZoomInst> t(kZoomInstances);
+#define CWT_ZOOM_ROW(I, QA, QB, QC, P, T, MINB, COST) \
+    t[I] = ZoomInst{QA, QA * QB * QC, ZoomCfg<QA, QB, QC, P, T, MINB>::NB, P, T, ZoomCfg<QA, QB, QC, P, T, MINB>::LAST, COST};
+        CWT_ZOOM_ALL(CWT_ZOOM_ROW)
+#undef CWT_ZOOM_ROW
+        return t;
+    }();
+    return table[(size_t)i];
+}
+
+}  // namespace
+
+#define CWT_ZOOM_DECLARE(I, QA, QB, QC, P, T, MINB, COST) \
+    template <>                                           \
+    const void *zoom_entry<I>(int mode);
+CWT_ZOOM_ALL(CWT_ZOOM_DECLARE)
+#undef CWT_ZOOM_DECLARE
+
+namespace {
+
+const void *kernel_of(int i, int mode) {
+    switch (i) {
+#define CWT_ZOOM_CASE(I, QA, QB, QC, P, T, MINB, COST) \
+    case I: return zoom_entry<I>(mode);
+        CWT_ZOOM_ALL(CWT_ZOOM_CASE)
+#undef CWT_ZOOM_CASE
+        default: return nullptr;
+    }
+}
+
+int smem_of(int i, int rows) {
+    switch (i) {
+#define CWT_ZOOM_CASE(I, QA, QB, QC, P, T, MINB, COST) \
+    case I: return ZoomCfg<QA, QB, QC, P, T, MINB>::smem(rows);
+        CWT_ZOOM_ALL(CWT_ZOOM_CASE)
+#undef CWT_ZOOM_CASE
+        default: return 0;
+    }
+}
+
+int row_smem_of(int i, int nr, int rs, int R) {
+    switch (i) {
+#define CWT_ZOOM_CASE(I, QA, QB, QC, P, T, MINB, COST) \
+    case I: return zoom_row_smem<ZoomCfg<QA, QB, QC, P, T, MINB>>(nr, rs, R);
+        CWT_ZOOM_ALL(CWT_ZOOM_CASE)
+#undef CWT_ZOOM_CASE
+        default: return 0;
+    }
+}
+
+constexpr int kMaxSmem = 227 * 1024;
+
+// Rows that P consecutive columns, the first a multiple of P, can meet.
+int rows_met(int P, int R) {
+    if (R % P == 0) return 1;
+    return P % R == 0 ? P / R : (P - 2) / R + 2;
+}
+
+// Slots of a tile row: consecutive rows of few residues start in consecutive banks.
+int row_stride(int M, int R) { return R < 16 ? M + ((R - M) & 15) : M; }
+
+// Rows per CTA of zoom_row_kernel: the most threads at work on a tile of about
+// 5000 points (several CTAs per SM), up to 8400.
+int rows_per_cta(int i, int M, int R) {
+    const int T = inst(i).T;
+    int best = 1;
+    double score = -1;
+    for (int nr = 1; nr * R <= T && (nr == 1 || nr * M <= 8400); ++nr) {
+        const int C = nr * R;
+        double v = (double)(T / C * C) / T;
+        if (nr * M < 4000) v *= nr * M / 4000.0;
+        if (nr * M > 5600) v *= 0.95;
+        if (v > score) score = v, best = nr;
+    }
+    return best;
+}
+
+// Opt instance i (mode) into the largest shared memory, once per device.
+cudaError_t ensure_zoom_smem(int i, int mode) {
+    static std::atomic<unsigned> done[kZoomInstances][3];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::atomic<unsigned> &d = done[i][mode];
+    if (dev < 32 && (d.load(std::memory_order_acquire) & (1u << dev))) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel_of(i, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess && dev < 32) d.fetch_or(1u << dev, std::memory_order_acq_rel);
+    return e;
+}
+
+// Cost of one row (ps) on instance i by columns.  A run of R outputs starts at
+// a multiple of R past the row's base: unless 8 divides both, its ends share
+// 32-byte sectors with runs stored by other instructions, and sectors written
+// in part cost L2 a read once the outputs of a launch exceed it (complex and
+// power of 32 Mi points, 8 x 16: 2.02 ps per point at R = 64, 2.09 at 40, 3.29
+// at 50, 3.68 at 63; 16 x 16: 2.16, 2.29, 4.03, 4.52).  Column groups that
+// meet several rows form more band products.
+double column_cost(int i, const ZoomShape &z, int S) {
+    const int R = z.M / inst(i).Q, P = inst(i).P;
+    const bool large = 64.0 * S * z.row_bytes > 192e6;  // at a nominal 64 channels
+    double f = 1.0;
+    if (P > 4 && (R % 8 != 0 || z.n_out % 8 != 0)) f = large ? (R % 4 == 0 && z.n_out % 4 == 0 ? 1.3 : 1.7) : 1.15;
+    if (P > 4 && R < 8) f = R % 4 == 0 ? 1.35 : 1.9;
+    if (R % P != 0 && P % R != 0) f *= 1.1;
+    if (z.sub != 1) f *= 1.4;  // a division per output
+    return (double)z.M * inst(i).cost * f;
+}
+
+// Cost of one row (ps) on instance i by whole rows: 1.12 of the column cost,
+// more where every row's band product serves few residues (8 x 16, power:
+// 1.74 ps per point at R = 32, 1.84 at 16, 1.88 at 8, 2.06 at 4, 2.57 at 2)
+// and where rows start off a sector, the more the fewer the slots of the last
+// pass (1.93, 2.07, 2.21, 2.57, 3.36).
+double whole_cost(int i, const ZoomShape &z) {
+    const int R = z.M / inst(i).Q, J = z.M / inst(i).LAST;
+    double f = 1.12 + 1.0 / R;
+    if (z.n_out % 8 != 0 || z.n_out == 0) f += 0.08 + 6.0 / J;
+    if (z.sub != 1) f *= 1.4;
+    return (double)z.M * inst(i).cost * f;
+}
+
+}  // namespace
+
+int zoom_class_L(const ZoomClass &c, int M) { return M / inst(c.inst).Q * inst(c.inst).QA; }
+
+void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomClass> *classes,
+                 std::vector<int4> *list, std::vector<int> *rest) {
+    classes->clear();
+    list->clear();
+    rest->clear();
+    // candidates: 2 i by columns, 2 i + 1 by whole rows; kRest the whole-row FFT kernels
+    constexpr int kRest = -1;
+    std::vector<int> open{kRest};
+    for (int i = 0; i < kZoomInstances; ++i) {
+        if (z.M % inst(i).Q != 0) continue;
+        const int R = z.M / inst(i).Q;
+        if (!z.rows_only && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem) open.push_back(2 * i);
+        if (!z.phase && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
+            row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(z.M, R), R) <= kMaxSmem)
+            open.push_back(2 * i + 1);
+    }
+    auto cost = [&](int k, int s) -> double {
+        if (k == kRest) return z.rest_cost;
+        const int i = k >> 1;
+        // the window starts at a multiple of NB
+        if (band[2 * s + 1] + band[2 * s] % inst(i).NB > inst(i).Q) return 1e30;
+        return (k & 1) ? whole_cost(i, z) : column_cost(i, z, S);
+    };
+    // every scale on its cheapest transform, then classes dissolved into the
+    // remaining ones while the launch they save (3 us) outweighs the dearer
+    // transforms of their scales, at a nominal 64 channels
+    auto assign = [&](const std::vector<int> &o, std::vector<int> *to) -> double {
+        double total = 0;
+        std::vector<char> used(o.size(), 0);
+        for (int s = 0; s < S; ++s) {
+            size_t b = o.size();
+            double c = 1e30;
+            for (size_t k = 0; k < o.size(); ++k) {
+                const double ck = cost(o[k], s);
+                if (ck < c) c = ck, b = k;
+            }
+            if (b == o.size()) return 1e300;
+            total += 64.0 * c;
+            used[b] = 1;
+            if (to) (*to)[(size_t)s] = o[b];
+        }
+        for (char u : used) total += u ? 3e6 : 0.0;
+        return total;
+    };
+    std::vector<int> to((size_t)S, kRest);
+    double total = assign(open, &to);
+    {
+        std::vector<int> u;
+        for (int k : open)
+            if (std::find(to.begin(), to.end(), k) != to.end()) u.push_back(k);
+        open = u;
+    }
+    while (open.size() > 1) {
+        double best = total;
+        size_t drop = open.size();
+        for (size_t k = 0; k < open.size(); ++k) {
+            std::vector<int> o = open;
+            o.erase(o.begin() + (long)k);
+            const double t = assign(o, nullptr);
+            if (t < best) best = t, drop = k;
+        }
+        if (drop == open.size()) break;
+        open.erase(open.begin() + (long)drop);
+        total = assign(open, &to);
+    }
+    for (int k : open) {
+        if (k == kRest) continue;
+        const int i = k >> 1, first = (int)list->size();
+        for (int s = 0; s < S; ++s)
+            if (to[(size_t)s] == k)
+                list->push_back(make_int4(s, band[2 * s], band[2 * s + 1], band[2 * s] / inst(i).NB * inst(i).NB));
+        if ((int)list->size() > first) classes->push_back({i, first, (int)list->size() - first, (k & 1) != 0});
+    }
+    for (int s = 0; s < S; ++s)
+        if (to[(size_t)s] == kRest) rest->push_back(s);
+    // the largest class first: the last launch's tail is then short
+    std::stable_sort(classes->begin(), classes->end(),
+                     [](const ZoomClass &a, const ZoomClass &b) { return a.ns > b.ns; });
+}
+
+cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const float2 *twl, const int4 *d_list,
+                        cudaStream_t st) {
+    const ZoomInst &t = inst(c.inst);
+    const int R = a.M / t.Q;
+    const long long rows = chans * c.ns;
+    if (rows >= 2147483647ll || rows * R >= 2147483647ll) return cudaErrorInvalidValue;
+    a.R = R;
+    a.L = R * t.QA;
+    a.twl = twl;
+    a.list = d_list + c.first;
+    a.ns = c.ns;
+    a.magM = zoom_magic((unsigned)a.M);
+    a.magSub = zoom_magic((unsigned)a.sub);
+    a.magL = zoom_magic((unsigned)a.L);
+    a.magR = zoom_magic((unsigned)R);
+    a.magNs = zoom_magic((unsigned)c.ns);
+    const int mode = c.rows ? 2 : a.oph || a.sub != 1 ? 1 : 0;
+    cudaError_t e = ensure_zoom_smem(c.inst, mode);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3((unsigned)t.T);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (c.rows) {
+        a.nr = rows_per_cta(c.inst, a.M, R);
+        a.nrows = (int)rows;
+        a.rs = row_stride(a.M, R);
+        const int J = a.M / t.LAST;  // last-pass slots of a row, and 7 for the shift
+        a.js = !a.epochs && a.n_out % 8 == 0 ? J : (J + 14) & ~7;
+        a.magC = zoom_magic((unsigned)(a.nr * R));
+        a.magJs = zoom_magic((unsigned)a.js);
+        a.magL2 = zoom_magic((unsigned)a.L);
+        cfg.gridDim = dim3((unsigned)((rows + a.nr - 1) / a.nr));
+        cfg.dynamicSmemBytes = (size_t)row_smem_of(c.inst, a.nr, a.rs, R);
+    } else {
+        a.cols = (unsigned)(rows * R);
+        a.rows = rows_met(t.P, R);
+        cfg.gridDim = dim3((a.cols + (unsigned)t.P - 1) / (unsigned)t.P);
+        cfg.dynamicSmemBytes = (size_t)smem_of(c.inst, a.rows);
+    }
+    void *params[] = {&a};
+    return cudaLaunchKernelExC(&cfg, kernel_of(c.inst, mode), params);
+}
+
+namespace {
+
+// Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
+// with kernels compiled at its creation takes the same split of its scales).
+double row_cost(const cwt_plan_s *p) {
+    if (!p->mr) return (double)p->M * (p->M <= kMaxFft ? 3.3 : 7.2);
+    if (p->cl > 1) return (double)p->N * (p->sch.fixed_cl >= 0 ? 7.2 : 30.0);
+    return (double)p->N * (p->sch.fixed >= 0 ? 3.4 : p->sch.fast >= 0 ? 6.0 : 14.0);
+}
+
+}  // namespace
+
+struct ZoomPlan {
+    std::vector<ZoomClass> classes;
+    std::vector<const float2 *> twl;  // per class: w_L^i, L = QA R
+    int4 *d_list = nullptr;
+    float2 *d_twl = nullptr;  // smooth lengths: those tables
+    int M = 0, sub = 1, tws = 1;
+    const float2 *tw = nullptr;
+};
+
+void free_zoom_plan(ZoomPlan *z) {
+    if (!z) return;
+    cudaFree(z->d_list);
+    cudaFree(z->d_twl);
+    delete z;
+}
+
+static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
+    const int S = p->S;
+    const int f = std::gcd(p->N, p->d), M = p->N / f;
+    std::vector<int> band(2 * (size_t)S);
+    cudaError_t e = cudaMemcpyAsync(band.data(), p->band, sizeof(int) * band.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    std::vector<ZoomClass> classes;
+    std::vector<int4> list;
+    std::vector<int> rest;
+    ZoomShape sh;
+    sh.N = p->N;
+    sh.M = M;
+    sh.sub = p->d / f;
+    sh.n_out = p->n_out;
+    sh.rest_cost = row_cost(p);
+    sh.phase = (p->outputs & CWT_OUT_PHASE) != 0;
+    sh.rows_only = false;
+    sh.row_bytes = (double)p->n_out * (((p->outputs & CWT_OUT_COMPLEX) ? 8 : 0) + ((p->outputs & CWT_OUT_POWER) ? 4 : 0) +
+                                       ((p->outputs & CWT_OUT_PHASE) ? 4 : 0));
+    zoom_select(sh, S, band.data(), &classes, &list, &rest);
+    // columns and grids stay within 31 bits
+    for (const ZoomClass &c : classes)
+        if ((double)p->C * c.ns * (M / inst(c.inst).Q) >= 2147483647.0) list.clear();
+    if (list.empty()) return cudaSuccess;
+    ZoomPlan *z = new ZoomPlan;
+    p->zoom = z;  // freed with the plan, also on failure
+    z->classes = classes;
+    z->M = M;
+    z->sub = sh.sub;
+    z->tw = p->mr ? p->twN : twiddles_pow2(p->tw, M);
+    z->tws = p->mr ? p->N / M : 1;
+    e = dmalloc(&z->d_list, sizeof(int4) * list.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(z->d_list, list.data(), sizeof(int4) * list.size(), cudaMemcpyHostToDevice, st);
+    // the first pass's tables w_L: powers of two from the device's, others here
+    size_t total_l = 0, at = 0;
+    for (const ZoomClass &c : classes) total_l += (size_t)zoom_class_L(c, M);
+    if (e == cudaSuccess && p->mr) e = dmalloc(&z->d_twl, sizeof(float2) * total_l);
+    for (const ZoomClass &c : classes) {
+        const int L = zoom_class_L(c, M);
+        if (e == cudaSuccess && p->mr) e = make_twiddles_n(L, z->d_twl + at, st);
+        z->twl.push_back(p->mr ? z->d_twl + at : twiddles_pow2(p->tw, L));
+        at += (size_t)L;
+    }
+    if (e == cudaSuccess && !rest.empty()) {
+        e = dmalloc(&p->rest_list, sizeof(int) * rest.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(p->rest_list, rest.data(), sizeof(int) * rest.size(), cudaMemcpyHostToDevice, st);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    p->rest_scales = (int)rest.size();
+    p->bytes += sizeof(int4) * list.size() + sizeof(int) * rest.size() + (p->mr ? sizeof(float2) * total_l : 0);
+    return e;
+}
+
+cudaError_t zoom_plan_create(cwt_plan_s *p, cudaStream_t st) {
+    p->rest_scales = p->S;
+    if (p->io != CWT_DTYPE_F32 || p->precision != CWT_PREC_FP32) return cudaSuccess;
+    try {
+        return zoom_plan_build(p, st);
+    } catch (const std::bad_alloc &) {
+        return cudaErrorMemoryAllocation;
+    }
+}
+
+cudaError_t launch_scale_block_zoom(const cwt_plan_s *p, float2 *out_c, float *out_p, float *out_ph,
+                                    cudaStream_t st) {
+    const ZoomPlan *z = p->zoom;
+    ZoomArgs a = {};
+    a.spec = p->spec;
+    a.bank = p->bank;
+    a.tw = z->tw;
+    a.oc = out_c;
+    a.op = out_p;
+    a.oph = out_ph;
+    a.N = a.wn = p->N;
+    a.M = z->M;
+    a.tws = z->tws;
+    a.S = p->S;
+    a.n_out = p->n_out;
+    a.sub = z->sub;
+    a.n_keep = z->sub * (p->n_out - 1) + 1;
+    // Launches overlap (programmatic dependent launch): the first after the
+    // forward FFTs waits for them before it reads a spectrum; a later one may
+    // start when every CTA of the one before has passed that point, reads the
+    // spectra at once and waits at its end, so that the stream's order holds.
+    bool after = p->rest_scales > 0;  // the whole-row kernel before saw the forward FFTs complete
+    for (size_t k = 0; k < z->classes.size(); ++k) {
+        a.after = after;
+        after = true;
+        const cudaError_t e = zoom_launch(z->classes[k], a, p->C, z->twl[k], z->d_list, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace cwtk

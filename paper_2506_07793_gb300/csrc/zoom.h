@@ -1,0 +1,57 @@
+// zoom.h -- the host's view of the zoom_kernel instances (zoom.cuh,
+// zoom_list.h): which scales run on which instance, and the launch of one
+// class of scales (zoom.cu).  Used by plans (zoom.cu) and batches (batch.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <vector>
+
+#include "zoom.cuh"
+#include "zoom_list.h"
+
+namespace cwtk {
+
+// The kernel of instance I: zoom_kernel MODE 0 or 1, or (2) zoom_row_kernel
+// (zoom_inst_<g>.cu).
+template <int I>
+const void *zoom_entry(int mode);
+
+#define CWT_ZOOM_DEFINE(I, QA, QB, QC, P, T, MINB, COST)                        \
+    template <>                                                                 \
+    const void *zoom_entry<I>(int mode) {                                       \
+        using Z = ZoomCfg<QA, QB, QC, P, T, MINB>;                              \
+        return mode == 0   ? (const void *)&zoom_kernel<Z, 0>                   \
+               : mode == 1 ? (const void *)&zoom_kernel<Z, 1>                   \
+                           : (const void *)&zoom_row_kernel<Z>;                 \
+    }
+
+// Scales [first, first + ns) of a device list on one instance; rows: by
+// zoom_row_kernel.
+struct ZoomClass {
+    int inst, first, ns;
+    bool rows;
+};
+
+// What zoom_select decides from: a row of N bins on M points of which every
+// sub-th is kept, output rows of n_out samples (0: of any length), the cost of
+// a row (ps) on the kernels that take the rest, and whether the phase is asked
+// for.
+struct ZoomShape {
+    int N, M, sub, n_out;
+    double rest_cost;
+    bool phase, rows_only;
+    double row_bytes;  // output bytes of one row
+};
+
+// Splits S scales with bands band[2 s] (start), band[2 s + 1] (length) into
+// classes, their entries for the device in *list, and the rest.
+void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomClass> *classes,
+                 std::vector<int4> *list, std::vector<int> *rest);
+int zoom_class_L(const ZoomClass &c, int M);  // points of its first pass's table
+// Launch class c for `chans` channels: a holds the pointers, N, M, tws, S,
+// n_out, sub, n_keep, after and the batch's fields.
+cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const float2 *twl, const int4 *d_list,
+                        cudaStream_t st);
+
+}  // namespace cwtk

@@ -1,0 +1,9 @@
+// zoom_inst_7.cu -- instances of zoom_kernel, group 7 of zoom_list.h (a
+// translation unit of its own so that the groups compile in parallel).
+#include "zoom.h"
+
+namespace cwtk {
+
+CWT_ZOOM_GROUP_7(CWT_ZOOM_DEFINE)
+
+}  // namespace cwtk
