@@ -13,6 +13,7 @@
 // the same Stockham kernels), so the results match cwt_execute.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -43,10 +44,21 @@ __global__ void na_twiddle_kernel(float2 *tw) {
     }
 }
 
-// Eq. 3 (Morlet spectrum in Hz, alias-summed) in FP64, the same evaluation
-// order as the plan's generator so that the FP32 bank is identical.
-__device__ double na_alias_sum(int k, int N, double fs, double f, double sg) {
-    const double kappa = exp(-0.5 * sg * sg);
+// F and sigma of up to kNaInline scales travel as kernel arguments; longer
+// lists are copied into the scratch.
+constexpr int kNaInline = 128;
+struct NaScales {
+    double F[kNaInline], sig[kNaInline];
+};
+
+// Exponent of the larger of Eq. 3's two terms at u = nu / F (the second is the
+// admissibility term, kappa = exp(-sigma^2 / 2)).
+__device__ __forceinline__ float na_exponent(float u, float h) { return -h * (u * u + 1.f - 2.f * fmaxf(u, 0.f)); }
+
+// Eq. 3 (Morlet spectrum in Hz) in FP64 summed over aliases, in the plan
+// generator's order.  Terms e^40 below the bin's largest (exponent `top`) are
+// left out: together they are under 1e-15 of it.
+__device__ double na_alias_sum(int k, int N, double fs, double f, double sg, double kappa, double top) {
     const double reach = 40.0 * f / sg;
     const double base = (double)k / (double)N;
     const double q_lo = ceil(-reach / fs - base), q_hi = floor((f + reach) / fs - base);
@@ -54,80 +66,98 @@ __device__ double na_alias_sum(int k, int N, double fs, double f, double sg) {
     for (double q = q_lo; q <= q_hi; q += 1.0) {
         const double u = (base + q) * fs / f;
         const double a = u - 1.0;
-        double g = exp(-0.5 * sg * sg * a * a);
-        g -= kappa * exp(-0.5 * sg * sg * u * u);
+        const double e1 = -0.5 * sg * sg * a * a, e2 = -0.5 * sg * sg * u * u;
+        double g = 0.0;
+        if (e1 > top - 40.0) g = exp(e1);
+        if (e2 - 0.5 * sg * sg > top - 40.0) g -= kappa * exp(e2);
         v += g;
     }
     return v;
 }
 
-// grid (nblk, S): per-block partial sums of the squared alias sums.
+// One CTA per scale: the spectrum of its bins in FP64, normalised to unit
+// energy with the 1/N of the inverse FFT folded in, rounded to FP32, and its
+// band.  Bound by FP64 exponentials (the pipe retires a warp instruction in 16
+// cycles), so only bins whose exponent is within 42 of the scale's largest are
+// evaluated, once: the others are below 1e-10 of the peak (a band's limit)
+// and add under 1e-30 to the energy.  Where the peak itself comes out far
+// below its exponent (a carrier under the first bins, whose terms cancel) the
+// bound says nothing and every bin is evaluated.  40 scales at N = 2048: this
+// launch and the forward FFTs' in 9 us; two kernels that evaluated every bin
+// three times took 112 us.
 __global__ void __launch_bounds__(kNaThreads)
-na_bank_energy_kernel(int N, double fs, const double *__restrict__ F, const double *__restrict__ sig,
-                      double *__restrict__ partial) {
-    __shared__ double red[kNaThreads];
-    const int s = blockIdx.y;
-    const int k = blockIdx.x * kNaThreads + threadIdx.x;
-    const double v = k < N ? na_alias_sum(k, N, fs, F[s], sig[s]) : 0.0;
-    red[threadIdx.x] = v * v;
-    __syncthreads();
-    for (int w = kNaThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[(size_t)s * gridDim.x + blockIdx.x] = red[0];
-}
-
-// One CTA per scale: normalise to unit energy (1/N folded in), FP32 bank, band.
-__global__ void __launch_bounds__(kNaThreads)
-na_bank_finish_kernel(int N, int nblk, double fs, const double *__restrict__ F,
-                      const double *__restrict__ sig, const double *__restrict__ partial,
-                      float *__restrict__ bank, int *__restrict__ band) {
-    __shared__ double sd[kNaThreads];
+na_bank_kernel(int N, int S, double fs, const double *par, const __grid_constant__ NaScales inl,
+               float *__restrict__ bank, int *__restrict__ band) {
+    extern __shared__ double raw[];  // [N]
+    __shared__ double sd[kNaThreads], sm[kNaThreads];
     __shared__ int smin[kNaThreads], smax[kNaThreads];
-    const int s = blockIdx.x;
-    float *b = bank + (size_t)s * N;
-    if (threadIdx.x == 0) {
-        double e = 0.0;
-        for (int i = 0; i < nblk; ++i) e += partial[(size_t)s * nblk + i];
-        sd[0] = e;
-    }
-    __syncthreads();
-    const double energy = sd[0];
-    const double scale = energy > 0.0 ? 1.0 / sqrt((double)N * energy) : 0.0;
-    __syncthreads();
-    double mx = 0.0;
-    for (int k = threadIdx.x; k < N; k += kNaThreads) {
-        const double v = na_alias_sum(k, N, fs, F[s], sig[s]);
-        b[k] = (float)(v * scale);
-        mx = fmax(mx, fabs(v));
-    }
-    sd[threadIdx.x] = mx;
+    griddep_launch();
+    const int s = blockIdx.x, tid = threadIdx.x;
+    const double F = par ? par[s] : inl.F[s], sg = par ? par[S + s] : inl.sig[s];
+    const double kappa = exp(-0.5 * sg * sg);
+    const float h = (float)(0.5 * sg * sg), du = (float)(fs / F / N), uN = (float)(fs / F);
+    auto exponent = [&](int k) {  // the nearest aliases of bin k: nu in [0, fs) and [-fs, 0)
+        return fmaxf(na_exponent((float)k * du, h), na_exponent((float)k * du - uN, h));
+    };
+    float top = -INFINITY;
+    for (int k = tid; k < N; k += kNaThreads) top = fmaxf(top, exponent(k));
+    sd[tid] = top;
     __syncthreads();
     for (int w = kNaThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sd[threadIdx.x] = fmax(sd[threadIdx.x], sd[threadIdx.x + w]);
+        if (tid < w) sd[tid] = fmax(sd[tid], sd[tid + w]);
         __syncthreads();
     }
-    const double thr = sd[0] * kBandRelThreshold;
+    const double peak = sd[0];
+    double energy = 0.0, mx = 0.0;
+    for (int all = 0;; ++all) {
+        __syncthreads();
+        double e = 0.0, m = 0.0;
+        for (int k = tid; k < N; k += kNaThreads) {
+            const float x = exponent(k);
+            double v = 0.0;
+            if (all || x > (float)peak - 42.f) v = na_alias_sum(k, N, fs, F, sg, kappa, all ? -1e300 : (double)x);
+            raw[k] = v;
+            e += v * v;
+            m = fmax(m, fabs(v));
+        }
+        sd[tid] = e;
+        sm[tid] = m;
+        __syncthreads();
+        for (int w = kNaThreads / 2; w > 0; w >>= 1) {
+            if (tid < w) {
+                sd[tid] += sd[tid + w];
+                sm[tid] = fmax(sm[tid], sm[tid + w]);
+            }
+            __syncthreads();
+        }
+        energy = sd[0];
+        mx = sm[0];
+        if (all || mx > exp(peak - 14.0)) break;
+    }
+    const double scale = energy > 0.0 ? 1.0 / sqrt((double)N * energy) : 0.0;
+    const double thr = mx * kBandRelThreshold;
+    float *b = bank + (size_t)s * N;
     int lo = N, hi = -N;
-    for (int k = threadIdx.x; k < N; k += kNaThreads) {
-        if (fabs(na_alias_sum(k, N, fs, F[s], sig[s])) > thr) {
+    for (int k = tid; k < N; k += kNaThreads) {
+        const double v = raw[k];
+        b[k] = (float)(v * scale);
+        if (fabs(v) > thr) {
             const int ks = k < N / 2 ? k : k - N;
             lo = min(lo, ks);
             hi = max(hi, ks);
         }
     }
-    smin[threadIdx.x] = lo;
-    smax[threadIdx.x] = hi;
+    smin[tid] = lo;
+    smax[tid] = hi;
     __syncthreads();
     for (int w = kNaThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            smin[threadIdx.x] = min(smin[threadIdx.x], smin[threadIdx.x + w]);
-            smax[threadIdx.x] = max(smax[threadIdx.x], smax[threadIdx.x + w]);
+        if (tid < w) {
+            smin[tid] = min(smin[tid], smin[tid + w]);
+            smax[tid] = max(smax[tid], smax[tid + w]);
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         int start = 0, len = 0;
         if (smax[0] >= smin[0]) {
             start = smin[0] < 0 ? smin[0] + N : smin[0];
@@ -144,6 +174,7 @@ na_forward_kernel(const float *__restrict__ x, int C, int n, float2 *__restrict_
                   const float2 *__restrict__ tw) {
     using RC = RowConfig<N>;
     extern __shared__ float2 na_smem[];
+    griddep_launch();
     const int rl = threadIdx.x / RC::T, j = threadIdx.x % RC::T;
     const int row = blockIdx.x * RC::ROWS + rl;
     const bool act = row < C;
@@ -155,6 +186,7 @@ na_forward_kernel(const float *__restrict__ x, int C, int n, float2 *__restrict_
         if (act) out[t] = v;
     };
     fft_row<N, RC::R, -1>(sm, tw, j, load, store);
+    griddep_wait();  // the bank, which this kernel overlaps: the stream's order holds
 }
 
 __device__ __noinline__ void na_store_phase(float *dst, float2 v) { *dst = phase_atan2(v.y, v.x); }
@@ -171,6 +203,7 @@ na_scale_block_kernel(const float2 *__restrict__ spec, const float *__restrict__
     const bool act = row < rows;
     const int c = act ? row / S : 0;
     const int s = act ? row - c * S : 0;
+    griddep_wait();  // bank and spectra
     float2 *sm = na_smem + rl * FftShape<N, RC::R>::SMEM_F2;
     const float2 *X = spec + (size_t)c * N;
     const float *W = bank + (size_t)s * N;
@@ -194,30 +227,30 @@ na_scale_block_kernel(const float2 *__restrict__ spec, const float *__restrict__
 }
 
 template <int N>
-cudaError_t na_run(const float *x, int C, int n, int S, char *base, size_t off_par, size_t off_part,
-                   size_t off_band, size_t off_bank, size_t off_spec, double fs, float2 *oc,
-                   float *op, float *oph, cudaStream_t st) {
+cudaError_t na_run(const float *x, int C, int n, int S, char *base, const double *par, const NaScales &inl,
+                   size_t off_band, size_t off_bank, size_t off_spec, double fs, float2 *oc, float *op, float *oph,
+                   cudaStream_t st) {
     using RC = RowConfig<N>;
-    static std::atomic<unsigned> attr_f{0}, attr_s{0};
-    cudaError_t e = ensure_smem_attr(na_forward_kernel<N>, RC::SMEM_BYTES, &attr_f);
+    static std::atomic<unsigned> attr_b{0}, attr_f{0}, attr_s{0};
+    cudaError_t e = ensure_smem_attr(na_bank_kernel, kMaxFft * (int)sizeof(double), &attr_b);
+    if (e == cudaSuccess) e = ensure_smem_attr(na_forward_kernel<N>, RC::SMEM_BYTES, &attr_f);
     if (e == cudaSuccess) e = ensure_smem_attr(na_scale_block_kernel<N>, RC::SMEM_BYTES, &attr_s);
     if (e != cudaSuccess) return e;
     const float2 *tw = (const float2 *)base;
-    const double *F = (const double *)(base + off_par);
-    const double *sig = F + S;
-    double *partial = (double *)(base + off_part);
     int *band = (int *)(base + off_band);
     float *bank = (float *)(base + off_bank);
     float2 *spec = (float2 *)(base + off_spec);
-    const int nblk = (N + kNaThreads - 1) / kNaThreads;
-    na_bank_energy_kernel<<<dim3(nblk, S), kNaThreads, 0, st>>>(N, fs, F, sig, partial);
-    na_bank_finish_kernel<<<S, kNaThreads, 0, st>>>(N, nblk, fs, F, sig, partial, bank, band);
-    na_forward_kernel<N><<<(C + RC::ROWS - 1) / RC::ROWS, RC::THREADS, RC::SMEM_BYTES, st>>>(
-        x, C, n, spec, tw);
+    na_bank_kernel<<<S, kNaThreads, N * (int)sizeof(double), st>>>(N, S, fs, par, inl, bank, band);
+    e = cudaGetLastError();
+    // the forward FFTs run beside the bank, the rows wait for both
+    if (e == cudaSuccess)
+        e = launch_dependent(na_forward_kernel<N>, (C + RC::ROWS - 1) / RC::ROWS, RC::THREADS, RC::SMEM_BYTES, st, x, C,
+                             n, spec, tw);
     const int rows = C * S;
-    na_scale_block_kernel<N><<<(rows + RC::ROWS - 1) / RC::ROWS, RC::THREADS, RC::SMEM_BYTES, st>>>(
-        spec, bank, band, tw, S, rows, n, oc, op, oph);
-    return cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_dependent(na_scale_block_kernel<N>, (rows + RC::ROWS - 1) / RC::ROWS, RC::THREADS, RC::SMEM_BYTES, st,
+                             (const float2 *)spec, (const float *)bank, (const int *)band, tw, S, rows, n, oc, op, oph);
+    return e;
 }
 
 std::mutex g_na_mutex;
@@ -290,20 +323,31 @@ extern "C" cwt_status cwt_execute_noalloc(const float *d_signal, int channels, i
     cudaStream_t st = (cudaStream_t)stream;
     char *base = nullptr;
     cudaError_t e = na_setup(dev, st, &base);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(base + off_par, freqs_hz, sizeof(double) * n_freqs,
-                            cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(base + off_par + sizeof(double) * n_freqs, n_cycles,
-                            sizeof(double) * n_freqs, cudaMemcpyHostToDevice, st);
+    // not inside a stream capture (see cwt.h), whether or not anything is copied
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return CWT_ECUDA;
+    NaScales inl;
+    const double *par = nullptr;
+    if (n_freqs <= kNaInline) {
+        std::copy(freqs_hz, freqs_hz + n_freqs, inl.F);
+        std::copy(n_cycles, n_cycles + n_freqs, inl.sig);
+    } else {
+        par = (const double *)(base + off_par);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(base + off_par, freqs_hz, sizeof(double) * n_freqs, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(base + off_par + sizeof(double) * n_freqs, n_cycles, sizeof(double) * n_freqs,
+                                cudaMemcpyHostToDevice, st);
+    }
     if (e == cudaSuccess) {
         float2 *oc = (float2 *)d_complex;
         const int S = n_freqs;
         switch (ilog2c(N)) {
 #define CWT_NA_CASE(L)                                                                             \
     case L:                                                                                        \
-        e = na_run<1 << L>(d_signal, channels, samples, S, base, off_par, off_part, off_band,     \
-                           off_bank, off_spec, fs, oc, d_power, d_phase, st);                      \
+        e = na_run<1 << L>(d_signal, channels, samples, S, base, par, inl, off_band, off_bank,    \
+                           off_spec, fs, oc, d_power, d_phase, st);                                \
         break;
             CWT_NA_CASE(5) CWT_NA_CASE(6) CWT_NA_CASE(7) CWT_NA_CASE(8) CWT_NA_CASE(9)
             CWT_NA_CASE(10) CWT_NA_CASE(11) CWT_NA_CASE(12) CWT_NA_CASE(13) CWT_NA_CASE(14)
