@@ -69,6 +69,7 @@ template <int N, typename IO, bool PLAIN>
 __global__ void __cluster_dims__(N / kClPoints, 1, 1) __launch_bounds__(kClThreads, 1)
 cl_scale_block_kernel(const ClArgs a) {
     using V2 = typename IO2c<IO>::type;
+    griddep_wait();  // the forward FFTs
     griddep_launch();
     extern __shared__ float2 clsm[];
     constexpr int CL = ClusterShape<N>::CL;
@@ -156,9 +157,8 @@ cudaError_t cl_sb_nk(const ClArgs &a, int rows, cudaStream_t st) {
     static std::atomic<unsigned> done{0};
     cudaError_t e = cl_attr(cl_scale_block_kernel<N, IO, PLAIN>, ClusterShape<N>::SMEM_BYTES, &done);
     if (e != cudaSuccess) return e;
-    cl_scale_block_kernel<N, IO, PLAIN>
-        <<<rows * ClusterShape<N>::CL, kClThreads, ClusterShape<N>::SMEM_BYTES, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(cl_scale_block_kernel<N, IO, PLAIN>, rows * ClusterShape<N>::CL, kClThreads,
+                            ClusterShape<N>::SMEM_BYTES, st, a);
 }
 
 template <int N, typename IO>

@@ -133,6 +133,24 @@ cudaError_t ensure_smem_attr(K *kernel, int bytes, std::atomic<unsigned> *done) 
     return e;
 }
 
+// Launch k as a programmatic dependent of the kernel before it on `st`: its CTAs
+// may start while that one finishes, and wait for its results at griddep_wait
+// (fft_core.cuh).  Hides the launch gap between a transform's kernels.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*k)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Host-side check of the wavelet kind and its shape parameters (n_cycles
 // already checked > 0 and finite): Morlet/Gabor take sigma = n_cycles; the
 // generalized Morse wavelet takes beta = n_cycles <= 1000 and 0 < gamma <= 64.

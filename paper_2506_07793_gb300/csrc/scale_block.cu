@@ -50,7 +50,6 @@ scale_block_kernel(const SBArgs a) {
     using RC = RowConfig<M>;
     using V2 = typename IO2<IO>::type;
     extern __shared__ float2 smem2[];
-    griddep_launch();
     const int rl = threadIdx.x / RC::T, j = threadIdx.x % RC::T;
     const int row = blockIdx.x * RC::ROWS + rl;
     const bool act = row < a.rows;
@@ -69,6 +68,8 @@ scale_block_kernel(const SBArgs a) {
     // wider than M (always for fold 1), at most one k qualifies:
     // k = b0 + ((j - b0) mod M).
     const bool narrow = B <= M;
+    griddep_wait();  // the forward FFTs
+    griddep_launch();
     auto load = [&](int jj) -> float2 {
         float2 acc = make_float2(0.f, 0.f);
         if (fold == 1) {  // k = jj: addresses stay base + constant offsets
@@ -153,8 +154,7 @@ cudaError_t sb_n(const SBArgs &a, cudaStream_t st) {
     cudaError_t e = ensure_smem_attr(scale_block_kernel<M, IO>, RC::SMEM_BYTES, &attr_done);
     if (e != cudaSuccess) return e;
     const int grid = (a.rows + RC::ROWS - 1) / RC::ROWS;
-    scale_block_kernel<M, IO><<<grid, RC::THREADS, RC::SMEM_BYTES, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(scale_block_kernel<M, IO>, grid, RC::THREADS, RC::SMEM_BYTES, st, a);
 }
 
 template <typename IO>

@@ -102,8 +102,8 @@ cudaError_t sb_launch(const cwt_plan_s *p, const ClMrArgs &a, cudaStream_t st, i
     if (e == cudaSuccess) e = ensure_cluster_attr<CL>(scale_block_kernel<CL, FX>, &done_cl);
     if (e != cudaSuccess) return e;
     const int threads = (p->sch.T + 31) & ~31;
-    scale_block_kernel<CL, FX><<<(rows < 0 ? p->C * a.ns : rows) * CL, threads, smem, st>>>(a, p->sch);
-    return cudaGetLastError();
+    return launch_dependent(scale_block_kernel<CL, FX>, (rows < 0 ? p->C * a.ns : rows) * CL, threads, smem, st, a,
+                            p->sch);
 }
 
 template <int CL, class FX>

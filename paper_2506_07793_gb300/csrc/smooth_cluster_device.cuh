@@ -154,6 +154,7 @@ __device__ __forceinline__ void cross(const float2 *sm, const float2 *__restrict
 template <int CL, class FX>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(max_threads<FX>(), min_blocks<FX>())
 scale_block_kernel(const ClMrArgs a, const MrSchedule sch) {
+    griddep_wait();  // the forward FFTs
     griddep_launch();
     extern __shared__ float2 mrsm[];
     float2 *sm = mrsm;

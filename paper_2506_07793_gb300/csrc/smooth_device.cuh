@@ -33,6 +33,7 @@ __device__ __noinline__ inline void mr_phase_d(double *dst, float2 v) { *dst = (
 template <bool LIN, typename RunRow>
 __device__ __forceinline__ void mr_sb_row(const MrArgs &a, int N, int T, int R0, const RowSlot &rs, int rows,
                                           const RunRow &run_row) {
+    griddep_wait();  // the forward FFTs
     griddep_launch();
     extern __shared__ float2 mrsm[];
     const int row = rs.active ? (int)blockIdx.x * rows + rs.rr : 0;

@@ -18,8 +18,7 @@ cudaError_t sb_launch(const MrArgs &a, cudaStream_t st) {
     cudaError_t e = ensure_smem_attr(mr_fixed_scale_block_kernel<FX>, smem, &done);
     if (e != cudaSuccess) return e;
     const int grid = (a.total_rows + FX::ROWS - 1) / FX::ROWS;
-    mr_fixed_scale_block_kernel<FX><<<grid, FX::THREADS, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(mr_fixed_scale_block_kernel<FX>, grid, FX::THREADS, smem, st, a);
 }
 
 template <class FX>

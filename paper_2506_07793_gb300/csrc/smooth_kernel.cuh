@@ -42,8 +42,8 @@ cudaError_t mr_sb_launch(const cwt_plan_s *p, const MrArgs &a, cudaStream_t st) 
     const int rows = mr_launch_rows(p->sch, a.total_rows);
     const int smem = rows * (p->N + (p->N >> 4)) * 8;
     const int threads = (rows * p->sch.T + 31) & ~31;
-    mr_scale_block_kernel<RA, RB><<<(a.total_rows + rows - 1) / rows, threads, smem, st>>>(a, p->sch, rows);
-    return cudaGetLastError();
+    return launch_dependent(mr_scale_block_kernel<RA, RB>, (a.total_rows + rows - 1) / rows, threads, smem, st, a, p->sch,
+                            rows);
 }
 
 // Forward FFT of each zero-padded channel (float32 or float64 samples), Eq. 2;
