@@ -21,6 +21,7 @@ constexpr int kMaxBatchLog2 = 13;              // N_e <= kTile
 struct BatchItem {
     long long in_off;   // element offset of channel c0 of the epoch in the packed input
     long long out_off;  // element offset of row (c0, scale 0) in each packed output
+    long long ws_off;   // element offset of channel c0's window of bins in the workspace
     int n;              // epoch length
     int log2n;          // log2 N_e
     int G;              // channels in this item
@@ -37,6 +38,11 @@ struct BatchArgs {
     int *counter;
     const float *bank[kMaxBatchLog2 + 1];  // per log2 N: [S][N]
     const int *band[kMaxBatchLog2 + 1];    // per log2 N: [S][2]
+    // per log2 N: the scales whose rows run here (null: all), how many, and the
+    // window of bins (start mod N, count) that the residue-class rows read
+    const int *rest[kMaxBatchLog2 + 1];
+    int nrest[kMaxBatchLog2 + 1], w0[kMaxBatchLog2 + 1], wn[kMaxBatchLog2 + 1];
+    float2 *ws;                            // those windows, [epoch][channel][wn]
     const float2 *tw;
     int S, d;
 };
@@ -114,7 +120,9 @@ __device__ __noinline__ void batch_inverse(const BatchArgs &a, const BatchItem &
     float *const oph = a.oph;
     const float2 *const tw = a.tw;
     const long long out_off = it.out_off;
-    const int rows = it.G * S;
+    const int ns = a.nrest[it.log2n];
+    const int *const list = a.rest[it.log2n];
+    const int rows = it.G * ns;
     const float *bank = a.bank[it.log2n];
     const int *band = a.band[it.log2n];
     const int nmask = N - 1;
@@ -126,8 +134,9 @@ __device__ __noinline__ void batch_inverse(const BatchArgs &a, const BatchItem &
     for (int r0 = 0; r0 < rows; r0 += P) {
         const int row = r0 + rl;
         const bool act = row < rows;
-        const int g = act ? row / S : 0;
-        const int s = act ? row - g * S : 0;
+        const int g = act ? row / ns : 0;
+        int s = act ? row - g * ns : 0;
+        if (list) s = list[s];
         const float2 *sp = spec + g * N;
         const float *W = bank + (size_t)s * N;
         const int b0 = band[2 * s], B = act ? band[2 * s + 1] : 0;
@@ -157,7 +166,7 @@ __device__ __noinline__ void batch_inverse(const BatchArgs &a, const BatchItem &
             }
             return acc;
         };
-        const long long obase = out_off + (long long)row * n_out;
+        const long long obase = out_off + (long long)(g * S + s) * n_out;
         auto store = [&](int t, float2 v) {
             if (!act) return;
             int o = t;
@@ -218,7 +227,13 @@ __global__ void __launch_bounds__(kBThreads, 2) batch_kernel(const BatchArgs a) 
             default: break;
         }
         __syncthreads();  // spectra complete before any row reads them
-        batch_inverse_dispatch<RI>(a, it, spec, stage);
+        if (const int wn = a.wn[it.log2n]) {
+            const int N = 1 << it.log2n, w0 = a.w0[it.log2n];
+            for (int g = 0; g < it.G; ++g)
+                for (int i = threadIdx.x; i < wn; i += kBThreads)
+                    a.ws[it.ws_off + (long long)g * wn + i] = *CWT_SMEM(&spec[g * N + ((w0 + i) & (N - 1))]);
+        }
+        if (a.nrest[it.log2n]) batch_inverse_dispatch<RI>(a, it, spec, stage);
         __syncthreads();  // s_item and the spectra are free again
     }
 }

@@ -174,41 +174,42 @@ inline bool wavelet_params_ok(int wavelet, const double *n_cycles, int n, double
 // the exact alias-summed closed form.
 constexpr double kMinSpectrumPeak = 1e-150;
 
-// Largest |P[k]| over the bins that can hold the maximum of a scale's
-// alias-summed spectrum (Eq. 3/4 for Morlet/Gabor with sig = sigma, Eq. 5 for
-// the GMW with sig = beta): the two bins around the carrier F and the bins
-// 0, 1 and N - 1 around DC, with the aliases q = -2..2.  Host-only.
-inline double spectrum_peak_on_grid(int wavelet, double F, double sig, double gamma, double fs,
-                                    int N) {
+// Whether the scale's alias-summed spectrum (Eq. 3/4 for Morlet/Gabor with sig
+// = sigma, Eq. 5 for the GMW with sig = beta) reaches kMinSpectrumPeak on a bin
+// that can hold its maximum: the two bins around the carrier F and the bins 0,
+// 1 and N - 1 around DC, with the aliases q = -2..2; the first such bin settles
+// it (for an ordinary scale the carrier's: 10 exponentials instead of 50).
+// Host-only.
+inline bool spectrum_on_grid(int wavelet, double F, double sig, double gamma, double fs, int N) {
+    const bool gmw = wavelet == CWT_WAVELET_GMW;
+    const double kappa = wavelet == CWT_WAVELET_MORLET ? std::exp(-0.5 * sig * sig) : 0.0;
+    const double wp = gmw ? std::pow(sig / gamma, 1.0 / gamma) : 0.0;
+    const double la = gmw ? std::log(2.0) + (sig / gamma) * (1.0 + std::log(gamma) - std::log(sig)) : 0.0;
     auto g = [&](double nu) -> double {
-        if (wavelet == CWT_WAVELET_GMW) {
+        if (gmw) {
             if (!(nu > 0.0)) return 0.0;
-            const double wp = std::pow(sig / gamma, 1.0 / gamma);
             const double w = wp * nu / F;
-            const double la = std::log(2.0) + (sig / gamma) * (1.0 + std::log(gamma) - std::log(sig));
             return std::exp(la + sig * std::log(w) - std::pow(w, gamma));
         }
-        const double kappa = wavelet == CWT_WAVELET_GABOR ? 0.0 : std::exp(-0.5 * sig * sig);
         const double u = nu / F;
         return std::exp(-0.5 * sig * sig * (u - 1.0) * (u - 1.0)) - kappa * std::exp(-0.5 * sig * sig * u * u);
     };
     const long long k0 = (long long)std::floor(F * (double)N / fs);
-    const long long ks[5] = {0, 1, N - 1, k0, k0 + 1};
-    double best = 0.0;
+    const long long ks[5] = {k0, k0 + 1, 0, 1, N - 1};
     for (long long k : ks) {
         const long long kk = ((k % N) + N) % N;
         double sum = 0.0;
         for (int q = -2; q <= 2; ++q) sum += g(((double)kk / (double)N + q) * fs);
-        best = std::max(best, std::fabs(sum));
+        if (std::fabs(sum) >= kMinSpectrumPeak) return true;
     }
-    return best;
+    return false;
 }
 
 // True when every scale passes the check above at length N.
 inline bool scales_on_grid(int wavelet, const double *F, const double *sig, int S, double gamma,
                            double fs, int N) {
     for (int s = 0; s < S; ++s)
-        if (!(spectrum_peak_on_grid(wavelet, F[s], sig[s], gamma, fs, N) >= kMinSpectrumPeak)) return false;
+        if (!spectrum_on_grid(wavelet, F[s], sig[s], gamma, fs, N)) return false;
     return true;
 }
 

@@ -58,18 +58,17 @@ __device__ __forceinline__ float na_exponent(float u, float h) { return -h * (u 
 // Eq. 3 (Morlet spectrum in Hz) in FP64 summed over aliases, in the plan
 // generator's order.  Terms e^40 below the bin's largest (exponent `top`) are
 // left out: together they are under 1e-15 of it.
-__device__ double na_alias_sum(int k, int N, double fs, double f, double sg, double kappa, double top) {
-    const double reach = 40.0 * f / sg;
-    const double base = (double)k / (double)N;
-    const double q_lo = ceil(-reach / fs - base), q_hi = floor((f + reach) / fs - base);
+__device__ __forceinline__ double na_alias_sum(double base, double r, double lo, double hi, double h, double kappa,
+                                               double top) {
+    const double q_lo = ceil(lo - base), q_hi = floor(hi - base);
     double v = 0.0;
     for (double q = q_lo; q <= q_hi; q += 1.0) {
-        const double u = (base + q) * fs / f;
+        const double u = (base + q) * r;
         const double a = u - 1.0;
-        const double e1 = -0.5 * sg * sg * a * a, e2 = -0.5 * sg * sg * u * u;
+        const double e1 = -h * a * a, e2 = -h * u * u;
         double g = 0.0;
         if (e1 > top - 40.0) g = exp(e1);
-        if (e2 - 0.5 * sg * sg > top - 40.0) g -= kappa * exp(e2);
+        if (e2 - h > top - 40.0) g -= kappa * exp(e2);
         v += g;
     }
     return v;
@@ -78,9 +77,9 @@ __device__ double na_alias_sum(int k, int N, double fs, double f, double sg, dou
 // One CTA per scale: the spectrum of its bins in FP64, normalised to unit
 // energy with the 1/N of the inverse FFT folded in, rounded to FP32, and its
 // band.  Bound by FP64 exponentials (the pipe retires a warp instruction in 16
-// cycles), so only bins whose exponent is within 42 of the scale's largest are
-// evaluated, once: the others are below 1e-10 of the peak (a band's limit)
-// and add under 1e-30 to the energy.  Where the peak itself comes out far
+// cycles), so only bins whose exponent is within 27 of the scale's largest are
+// evaluated, once, and no other takes an FP64 instruction: the others are at
+// 2e-12 of the peak (a band's limit is 1e-10) and add under 1e-19 to the energy.  Where the peak itself comes out far
 // below its exponent (a carrier under the first bins, whose terms cancel) the
 // bound says nothing and every bin is evaluated.  40 scales at N = 2048: this
 // launch and the forward FFTs' in 9 us; two kernels that evaluated every bin
@@ -94,31 +93,36 @@ na_bank_kernel(int N, int S, double fs, const double *par, const __grid_constant
     griddep_launch();
     const int s = blockIdx.x, tid = threadIdx.x;
     const double F = par ? par[s] : inl.F[s], sg = par ? par[S + s] : inl.sig[s];
-    const double kappa = exp(-0.5 * sg * sg);
-    const float h = (float)(0.5 * sg * sg), du = (float)(fs / F / N), uN = (float)(fs / F);
+    const double hh = 0.5 * sg * sg, kappa = exp(-hh), r = fs / F, rN = 1.0 / (double)N;  // N is a power of two
+    const double reach = 40.0 * F / sg, q_min = -reach / fs, q_max = (F + reach) / fs;
+    const float h = (float)hh, du = (float)(r * rN), uN = (float)r;
     auto exponent = [&](int k) {  // the nearest aliases of bin k: nu in [0, fs) and [-fs, 0)
         return fmaxf(na_exponent((float)k * du, h), na_exponent((float)k * du - uN, h));
     };
+    __shared__ float sf[kNaThreads];
     float top = -INFINITY;
     for (int k = tid; k < N; k += kNaThreads) top = fmaxf(top, exponent(k));
-    sd[tid] = top;
+    sf[tid] = top;
     __syncthreads();
     for (int w = kNaThreads / 2; w > 0; w >>= 1) {
-        if (tid < w) sd[tid] = fmax(sd[tid], sd[tid + w]);
+        if (tid < w) sf[tid] = fmaxf(sf[tid], sf[tid + w]);
         __syncthreads();
     }
-    const double peak = sd[0];
+    const float peak = sf[0];
+    float cut = peak - 27.f;
     double energy = 0.0, mx = 0.0;
-    for (int all = 0;; ++all) {
+    for (;;) {
         __syncthreads();
         double e = 0.0, m = 0.0;
         for (int k = tid; k < N; k += kNaThreads) {
             const float x = exponent(k);
-            double v = 0.0;
-            if (all || x > (float)peak - 42.f) v = na_alias_sum(k, N, fs, F, sg, kappa, all ? -1e300 : (double)x);
-            raw[k] = v;
-            e += v * v;
-            m = fmax(m, fabs(v));
+            if (x > cut) {
+                const double v = na_alias_sum((double)k * rN, r, q_min, q_max, hh, kappa,
+                                              cut > -INFINITY ? (double)x : -1e300);
+                raw[k] = v;
+                e += v * v;
+                m = fmax(m, fabs(v));
+            }
         }
         sd[tid] = e;
         sm[tid] = m;
@@ -132,20 +136,25 @@ na_bank_kernel(int N, int S, double fs, const double *par, const __grid_constant
         }
         energy = sd[0];
         mx = sm[0];
-        if (all || mx > exp(peak - 14.0)) break;
+        if (cut == -INFINITY || mx > exp((double)peak - 1.0)) break;
+        cut = -INFINITY;
     }
     const double scale = energy > 0.0 ? 1.0 / sqrt((double)N * energy) : 0.0;
     const double thr = mx * kBandRelThreshold;
     float *b = bank + (size_t)s * N;
     int lo = N, hi = -N;
     for (int k = tid; k < N; k += kNaThreads) {
-        const double v = raw[k];
-        b[k] = (float)(v * scale);
-        if (fabs(v) > thr) {
-            const int ks = k < N / 2 ? k : k - N;
-            lo = min(lo, ks);
-            hi = max(hi, ks);
+        float w = 0.f;
+        if (exponent(k) > cut) {
+            const double v = raw[k];
+            w = (float)(v * scale);
+            if (fabs(v) > thr) {
+                const int ks = k < N / 2 ? k : k - N;
+                lo = min(lo, ks);
+                hi = max(hi, ks);
+            }
         }
+        b[k] = w;
     }
     smin[tid] = lo;
     smax[tid] = hi;

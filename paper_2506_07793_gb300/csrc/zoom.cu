@@ -86,8 +86,20 @@ int rows_met(int P, int R) {
     return P % R == 0 ? P / R : (P - 2) / R + 2;
 }
 
-// Slots of a tile row: consecutive rows of few residues start in consecutive banks.
-int row_stride(int M, int R) { return R < 16 ? M + ((R - M) & 15) : M; }
+// Slots of one position of a tile row (QA R and padding) and of a tile row.  A
+// half-warp of the first pass that spans several rows, or the positions of
+// several threads, then falls into different banks: rows start R and a
+// thread's next NB positions nr R slots further, mod 16.
+int position_stride(int i, int nr, int R) {
+    const int C = nr * R, len = inst(i).QA * R;
+    if (C >= 16) return len;
+    const int nb = inst(i).NB, want = C / nb, mod = 16 / nb;
+    return len + (((want - len) % mod) + mod) % mod;
+}
+int row_stride(int i, int nr, int R) {
+    const int len = inst(i).Q / inst(i).QA * position_stride(i, nr, R);
+    return R < 16 && nr > 1 ? len + ((R - len) & 15) : len;
+}
 
 // Rows per CTA of zoom_row_kernel: the most threads at work on a tile of about
 // 5000 points (several CTAs per SM), up to 8400.
@@ -127,7 +139,7 @@ cudaError_t ensure_zoom_smem(int i, int mode) {
 // meet several rows form more band products.
 double column_cost(int i, const ZoomShape &z, int S) {
     const int R = z.M / inst(i).Q, P = inst(i).P;
-    const bool large = 64.0 * S * z.row_bytes > 192e6;  // at a nominal 64 channels
+    const bool large = z.channels * S * z.row_bytes > 192e6;
     double f = 1.0;
     if (P > 4 && (R % 8 != 0 || z.n_out % 8 != 0)) f = large ? (R % 4 == 0 && z.n_out % 4 == 0 ? 1.3 : 1.7) : 1.15;
     if (P > 4 && R < 8) f = R % 4 == 0 ? 1.35 : 1.9;
@@ -164,9 +176,10 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
     for (int i = 0; i < kZoomInstances; ++i) {
         if (z.M % inst(i).Q != 0) continue;
         const int R = z.M / inst(i).Q;
-        if (!z.rows_only && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem) open.push_back(2 * i);
-        if (!z.phase && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
-            row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(z.M, R), R) <= kMaxSmem)
+        // few residues leave a row's band product little use and its stores short
+        if (!z.rows_only && (R >= 4 || inst(i).P <= 4) && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem) open.push_back(2 * i);
+        if (!z.phase && R >= 2 && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
+            row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(i, rows_per_cta(i, z.M, R), R), R) <= kMaxSmem)
             open.push_back(2 * i + 1);
     }
     auto cost = [&](int k, int s) -> double {
@@ -178,7 +191,7 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
     };
     // every scale on its cheapest transform, then classes dissolved into the
     // remaining ones while the launch they save (3 us) outweighs the dearer
-    // transforms of their scales, at a nominal 64 channels
+    // transforms of their scales, at a nominal number of channels
     auto assign = [&](const std::vector<int> &o, std::vector<int> *to) -> double {
         double total = 0;
         std::vector<char> used(o.size(), 0);
@@ -190,7 +203,7 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
                 if (ck < c) c = ck, b = k;
             }
             if (b == o.size()) return 1e300;
-            total += 64.0 * c;
+            total += z.channels * c;
             used[b] = 1;
             if (to) (*to)[(size_t)s] = o[b];
         }
@@ -263,7 +276,8 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     if (c.rows) {
         a.nr = rows_per_cta(c.inst, a.M, R);
         a.nrows = (int)rows;
-        a.rs = row_stride(a.M, R);
+        a.ps = position_stride(c.inst, a.nr, R);
+        a.rs = row_stride(c.inst, a.nr, R);
         const int J = a.M / t.LAST;  // last-pass slots of a row, and 7 for the shift
         a.js = !a.epochs && a.n_out % 8 == 0 ? J : (J + 14) & ~7;
         a.magC = zoom_magic((unsigned)(a.nr * R));
@@ -327,6 +341,7 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     sh.rest_cost = row_cost(p);
     sh.phase = (p->outputs & CWT_OUT_PHASE) != 0;
     sh.rows_only = false;
+    sh.channels = 64;
     sh.row_bytes = (double)p->n_out * (((p->outputs & CWT_OUT_COMPLEX) ? 8 : 0) + ((p->outputs & CWT_OUT_POWER) ? 4 : 0) +
                                        ((p->outputs & CWT_OUT_PHASE) ? 4 : 0));
     zoom_select(sh, S, band.data(), &classes, &list, &rest);

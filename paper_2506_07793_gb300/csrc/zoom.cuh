@@ -51,9 +51,10 @@ struct ZoomArgs {
     int rows;            // most rows that one CTA's columns meet
     int sub, n_keep;     // outputs t = sub o, o < n_out; n_keep = sub (n_out - 1) + 1
     int after;           // 1: the spectra are complete when this kernel starts (see zoom.cu)
-    // zoom_row_kernel: rows per CTA and of the launch, slots of a tile row and
-    // of a row's last pass, zoom_magic of nr R, the slots, QA R and sub
-    int nr, nrows, rs, js;
+    // zoom_row_kernel: rows per CTA and of the launch, slots of a tile row, of
+    // one position of it (QA R and padding) and of a row's last pass, zoom_magic
+    // of nr R, the last pass's slots, QA R and sub
+    int nr, nrows, rs, ps, js;
     unsigned magC, magJs, magL2, magSub;
     // batches: channel c is channel c mod C of epoch c / C (null: one epoch);
     // its spectrum holds the wn bins from w0 mod N (0 and N without epochs)
@@ -100,8 +101,8 @@ struct ZoomCfg {
 };
 
 // The band product Y[k] = X[k] W[k] of a row by k mod Q, over the window
-// [sc.w, sc.w + Q) of bins; X holds bins [w0, w0 + ...) mod N.  Threads
-// lane, lane + STEP, ... of the row take part.
+// [sc.w, sc.w + Q) of bins; X holds bins [w0, w0 + ...) mod N.  STEP threads
+// take part, `lane` among them.
 template <int Q, int STEP>
 __device__ __forceinline__ void zoom_fill(float2 *Y, int lane, const int4 &sc, const float2 *X, int w0, int wn,
                                           const float *W, int N) {
@@ -153,6 +154,23 @@ template <int R>
 __device__ __forceinline__ float2 zoom_w8(const float2 *tw, unsigned i, unsigned M, unsigned magM, int tws) {
     if constexpr (R > 8) return __ldg(&tw[zoom_mod(8u * i, M, magM) * (unsigned)tws]);
     else return make_float2(1.f, 0.f);
+}
+
+// fill(row, lane, int_c<threads of the row>) for each of n rows: all T threads
+// one row after the other when there are few (each costs a load latency), a
+// warp per row, or 8 threads.
+template <int T, typename F>
+__device__ __forceinline__ void zoom_rows(int n, int tid, const F &fill) {
+    if (n < T / 32) {
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) fill(i, tid, int_c<T>{});
+    } else if (n <= T / 16) {
+#pragma unroll 1
+        for (int i = tid >> 5; i < n; i += T / 32) fill(i, tid & 31, int_c<32>{});
+    } else {
+#pragma unroll 1
+        for (int i = tid >> 3; i < n; i += T / 8) fill(i, tid & 7, int_c<8>{});
+    }
 }
 
 // Stores f(v[m]), m < min(L, left), at dst + m step.
@@ -216,13 +234,13 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_kernel(const ZoomArgs a) {
     griddep_launch();
     // band products of the CTA's rows by k mod Q (spectra through L2: a CTA may
     // share its SM with the kernel that wrote other spectra to the same address)
-#pragma unroll 1
-    for (int il = 0; il < nrow; ++il) {
+    zoom_rows<T>(nrow, tid, [&](int il, int lane, auto step) {
         int ic, is;
         zoom_divmod((unsigned)(row0 + il), (unsigned)a.ns, a.magNs, ic, is);
         const int4 z = __ldg(&a.list[is]);
-        zoom_fill<Q, T>(Y + il * Z::YP, tid, z, a.spec + (size_t)ic * N, 0, N, a.bank + (size_t)z.x * N, N);
-    }
+        zoom_fill<Q, decltype(step)::value>(Y + il * Z::YP, lane, z, a.spec + (size_t)ic * N, 0, N,
+                                            a.bank + (size_t)z.x * N, N);
+    });
     __syncthreads();
     // first pass: DFT over p
     {
@@ -408,9 +426,8 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
     }
     if (!a.after) griddep_wait();  // the forward FFTs
     griddep_launch();
-    // band products of the rows by k mod Q: a warp per row when there are
-    // enough rows, else the whole CTA one row after the other
-    auto fill = [&](int il, int lane, auto step) {
+    // band products of the rows by k mod Q
+    zoom_rows<T>(nr, tid, [&](int il, int lane, auto step) {
         int ic, is;
         zoom_divmod((unsigned)min(row0 + il, last), (unsigned)a.ns, a.magNs, ic, is);
         const int4 z = __ldg(&a.list[is]);
@@ -421,14 +438,7 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
             X = a.spec + a.epochs[e].spec + (long long)ch * a.wn;
         }
         zoom_fill<Q, decltype(step)::value>(Y + il * Z::YP, lane, z, X, a.w0, a.wn, a.bank + (size_t)z.x * N, N);
-    };
-    if (nr >= T / 32) {
-#pragma unroll 1
-        for (int il = tid >> 5; il < nr; il += T / 32) fill(il, tid & 31, int_c<32>{});
-    } else {
-#pragma unroll 1
-        for (int il = 0; il < nr; ++il) fill(il, tid, int_c<T>{});
-    }
+    });
     __syncthreads();
     // first pass: DFT over p
     if (on) {
@@ -450,7 +460,7 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
                         e[p] = t;
                     }
             }
-            float2 *dst = tile + rl * a.rs + b * (QA * R) + r;
+            float2 *dst = tile + rl * a.rs + b * a.ps + r;
             if constexpr (NB == 2) {
                 float2 v[QA], u[QA];
 #pragma unroll
@@ -463,7 +473,7 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
                 dft_r<QA, +1>(u);
 #pragma unroll
                 for (int k = 0; k < QA; ++k) *CWT_SMEM(&dst[k * R]) = v[k];
-                dst += QA * R;
+                dst += a.ps;
 #pragma unroll
                 for (int k = 0; k < QA; ++k) *CWT_SMEM(&dst[k * R]) = u[k];
             } else {
@@ -482,18 +492,18 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
         if (on) {
 #pragma unroll 1
             for (int q = th; q < QC * QA; q += TP) {
-                const int k1 = q % QA;
-                float2 *x = tile + rl * a.rs + q * R + r;  // (b1 QA + k1) R + r
+                const int b1 = q / QA, k1 = q - b1 * QA;
+                float2 *x = tile + rl * a.rs + b1 * a.ps + k1 * R + r;
                 const int i = QC * (r + R * k1);
                 const float2 w = __ldg(&a.tw[i * a.tws]);
                 const float2 w8 = zoom_w8<QB>(a.tw, (unsigned)i, (unsigned)a.M, a.magM, a.tws);
                 float2 v[QB];
 #pragma unroll
-                for (int b = 0; b < QB; ++b) v[b] = *CWT_SMEM(&x[b * (QC * QA * R)]);
+                for (int b = 0; b < QB; ++b) v[b] = *CWT_SMEM(&x[b * (QC * a.ps)]);
                 zoom_twiddle<QB>(v, w, w8);
                 dft_r<QB, +1>(v);
 #pragma unroll
-                for (int k = 0; k < QB; ++k) *CWT_SMEM(&x[k * (QC * QA * R)]) = v[k];
+                for (int k = 0; k < QB; ++k) *CWT_SMEM(&x[k * (QC * a.ps)]) = v[k];
             }
         }
     }
@@ -509,16 +519,16 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
         if ((unsigned)t0 >= (unsigned)min(step, z.n_keep)) continue;
         const float2 w = __ldg(&a.tw[t0 * a.tws]);
         const float2 w8 = zoom_w8<LAST>(a.tw, (unsigned)t0, (unsigned)a.M, a.magM, a.tws);
-        int at = t0;  // slot of (k2, k1, r): QC k2 L1 + t0 mod L1
+        int at = t0;  // slot of (k2, k1, r): QC k2 ps + t0 mod L1
         if constexpr (K2 > 1) {
             int k2, tl;
             zoom_divmod((unsigned)t0, (unsigned)L1, a.magL2, k2, tl);
-            at = QC * k2 * L1 + tl;
+            at = QC * k2 * a.ps + tl;
         }
         const float2 *x = tile + il * a.rs + at;
         float2 v[LAST];
 #pragma unroll
-        for (int b = 0; b < LAST; ++b) v[b] = *CWT_SMEM(&x[b * L1]);
+        for (int b = 0; b < LAST; ++b) v[b] = *CWT_SMEM(&x[b * a.ps]);
         zoom_twiddle<LAST>(v, w, w8);
         dft_r<LAST, +1>(v);
         if (a.sub != 1) {  // every sub-th sample: output o = t / sub

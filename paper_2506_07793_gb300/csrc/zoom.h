@@ -41,6 +41,7 @@ struct ZoomShape {
     int N, M, sub, n_out;
     double rest_cost;
     bool phase, rows_only;
+    double channels;   // nominal, for the cost of a launch against that of its rows
     double row_bytes;  // output bytes of one row
 };
 
