@@ -50,12 +50,17 @@ scale_block_kernel(const SBArgs a) {
     using RC = RowConfig<M>;
     using V2 = typename IO2<IO>::type;
     extern __shared__ float2 smem2[];
+    griddep_wait();  // the forward FFTs
+    griddep_launch();
     const int rl = threadIdx.x / RC::T, j = threadIdx.x % RC::T;
     const int row = blockIdx.x * RC::ROWS + rl;
     const bool act = row < a.rows;
-    const int c = act ? row / a.ns : 0;
-    int s = act ? row - c * a.ns : 0;
-    if (a.list) s = a.list[s];
+    // double rows are never split by scale: their output row is `row`
+    constexpr bool kListed = sizeof(IO) == 4;
+    const int ns = kListed ? a.ns : a.S;
+    const int c = act ? row / ns : 0;
+    int s = act ? row - c * ns : 0;
+    if (kListed && a.list) s = a.list[s];
     float2 *sm = smem2 + rl * FftShape<M, RC::R>::SMEM_F2;
 
     const float2 *X = a.spec + (size_t)c * (size_t)a.N;
@@ -68,8 +73,6 @@ scale_block_kernel(const SBArgs a) {
     // wider than M (always for fold 1), at most one k qualifies:
     // k = b0 + ((j - b0) mod M).
     const bool narrow = B <= M;
-    griddep_wait();  // the forward FFTs
-    griddep_launch();
     auto load = [&](int jj) -> float2 {
         float2 acc = make_float2(0.f, 0.f);
         if (fold == 1) {  // k = jj: addresses stay base + constant offsets
@@ -102,7 +105,7 @@ scale_block_kernel(const SBArgs a) {
         return acc;
     };
 
-    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
+    const size_t obase = (size_t)(kListed ? c * a.S + s : row) * (size_t)a.n_out;
     V2 *oc = (V2 *)a.out_c;
     IO *op = (IO *)a.out_p;
     IO *oph = (IO *)a.out_ph;
