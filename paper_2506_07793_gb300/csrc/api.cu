@@ -105,11 +105,10 @@ cwt_status run_execute(cwt_plan_s *p, const void *sig, void *oc, void *op, void 
     cudaError_t e = prof_begin(p, CWT_KERNEL_FORWARD_FFT, st, &ev);
     if (e == cudaSuccess) e = cwtk::launch_forward(p, sig, st);
     const bool tc = p->precision != CWT_PREC_FP32;
-    if (e == cudaSuccess && tc) e = cwtk::launch_tc_row_bounds(p, st);
+    if (e == cudaSuccess && tc && p->rest_scales > 0) e = cwtk::launch_tc_row_bounds(p, st);
     if (e == cudaSuccess) e = prof_end(p, st, &ev);
     if (e == cudaSuccess) e = prof_begin(p, CWT_KERNEL_SCALE_BLOCK, st, &ev);
-    if (e == cudaSuccess)
-        e = tc ? cwtk::launch_scale_block_tc(p, oc, op, oph, st) : cwtk::launch_scale_block(p, oc, op, oph, st);
+    if (e == cudaSuccess) e = cwtk::launch_scale_block(p, oc, op, oph, st);
     if (e == cudaSuccess) e = prof_end(p, st, &ev);
     if (e != cudaSuccess) return fail_cuda(p, e);
     return check_after(p, st);

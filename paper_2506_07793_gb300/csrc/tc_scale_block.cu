@@ -39,7 +39,8 @@ struct TcArgs {
     const float *wl1;     // [S] sum_k |W_s[k]| over the band
     const float2 *tw;
     void *out_c, *out_p, *out_ph;
-    int S, n_out, sub;
+    const int *list;      // [ns] the scales to run, or null: all (ns = S)
+    int S, ns, n_out, sub;
 };
 
 // Exact power-of-two scale of one row (see the file comment).
@@ -55,7 +56,9 @@ template <int CL, class T, typename IO>
 __device__ __forceinline__ void tc_row(const TcArgs &a, float2 *sm, int row, int rank) {
     using V2 = typename TcIO2<IO>::type;
     constexpr int N = CL * kTcNL;
-    const int c = row / a.S, s = row - c * a.S;
+    const int c = row / a.ns;
+    int s = row - c * a.ns;
+    if (a.list) s = a.list[s];
     const float2 *X = a.spec + (size_t)c * N;
     const float *W = a.bank + (size_t)s * N;
     const int b0 = a.band[2 * s], B = a.band[2 * s + 1];
@@ -95,7 +98,7 @@ __device__ __forceinline__ void tc_row(const TcArgs &a, float2 *sm, int row, int
     __syncthreads();
     tc_fft16384<T, +1>(sm, tab, Bm <= Q, load, first);
 
-    const size_t obase = (size_t)row * (size_t)a.n_out;
+    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
     V2 *oc = (V2 *)a.out_c;
     IO *op = (IO *)a.out_p;
     IO *oph = (IO *)a.out_ph;
@@ -270,9 +273,11 @@ cudaError_t launch_scale_block_tc(const cwt_plan_s *p, void *out_c, void *out_p,
     a.out_p = out_p;
     a.out_ph = out_ph;
     a.S = p->S;
+    a.ns = p->rest_scales;
+    a.list = p->rest_list;
     a.n_out = p->n_out;
     a.sub = p->d;  // no spectral fold on this path
-    const int rows = p->C * p->S;
+    const int rows = p->C * a.ns;
     const int log2n = ilog2c(p->N);
     const bool bf = p->precision == CWT_PREC_TC_BF16;
     if (p->io == CWT_DTYPE_F64)

@@ -300,6 +300,7 @@ namespace {
 // Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
 // with kernels compiled at its creation takes the same split of its scales).
 double row_cost(const cwt_plan_s *p) {
+    if (p->precision != CWT_PREC_FP32) return (double)p->N * 10.0;  // tensor-core stages: 340 us per 1024 x 32768
     if (!p->mr) return (double)p->M * (p->M <= kMaxFft ? 3.3 : 7.2);
     if (p->cl > 1) return (double)p->N * (p->sch.fixed_cl >= 0 ? 7.2 : 30.0);
     return (double)p->N * (p->sch.fixed >= 0 ? 3.4 : p->sch.fast >= 0 ? 6.0 : 14.0);
@@ -382,7 +383,8 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
 
 cudaError_t zoom_plan_create(cwt_plan_s *p, cudaStream_t st) {
     p->rest_scales = p->S;
-    if (p->io != CWT_DTYPE_F32 || p->precision != CWT_PREC_FP32) return cudaSuccess;
+    // double outputs keep the whole-row kernels' bits
+    if (p->io != CWT_DTYPE_F32) return cudaSuccess;
     try {
         return zoom_plan_build(p, st);
     } catch (const std::bad_alloc &) {
