@@ -202,6 +202,7 @@ cudaError_t make_length(cwt_plan_s *p, int L, cudaStream_t st, BatchLength *out)
         // for 144 epochs of 8 channels at d = 5
         sh.phase = (p->outputs & CWT_OUT_PHASE) != 0 || sh.sub != 1;
         sh.rows_only = true;
+        sh.wide = false;
         sh.channels = 4096;  // epochs x channels
         sh.row_bytes = 0;
         zoom_select(sh, S, band.data(), &l.classes, &list, &rest);

@@ -45,6 +45,11 @@ const ZoomInst &inst(int i) {
     const void *zoom_entry<I>(int mode);
 CWT_ZOOM_ALL(CWT_ZOOM_DECLARE)
 #undef CWT_ZOOM_DECLARE
+#define CWT_WIDE_DECLARE(I, QB, QC, P, T, MINB) \
+    template <>                                 \
+    const void *wide_rest_entry<I>(int mode);
+CWT_WIDE_REST(CWT_WIDE_DECLARE)
+#undef CWT_WIDE_DECLARE
 
 namespace {
 
@@ -75,6 +80,40 @@ int row_smem_of(int i, int nr, int rs, int R) {
         CWT_ZOOM_ALL(CWT_ZOOM_CASE)
 #undef CWT_ZOOM_CASE
         default: return 0;
+    }
+}
+
+struct WideInst {
+    int QB, QC, P, T, smem;
+};
+
+int wide_radix(int i) {
+    static const int r[kWideFirst] = {
+#define CWT_WIDE_ROW(I, QA) QA,
+        CWT_WIDE_FIRST(CWT_WIDE_ROW)
+#undef CWT_WIDE_ROW
+    };
+    return r[i];
+}
+
+const WideInst &wide_rest(int i) {
+    static const std::vector<WideInst> table = [] {
+        std::vector<WideInst> t(kWideRest);
+#define CWT_WIDE_ROW(I, QB, QC, P, T, MINB) t[I] = WideInst{QB, QC, P, T, WideCfg<QB, QC, P, T, MINB>::SMEM};
+        CWT_WIDE_REST(CWT_WIDE_ROW)
+#undef CWT_WIDE_ROW
+        return t;
+    }();
+    return table[(size_t)i];
+}
+
+const void *wide_kernel_of(int i, int mode) {
+    switch (i) {
+#define CWT_WIDE_CASE(I, QB, QC, P, T, MINB) \
+    case I: return wide_rest_entry<I>(mode);
+        CWT_WIDE_REST(CWT_WIDE_CASE)
+#undef CWT_WIDE_CASE
+        default: return nullptr;
     }
 }
 
@@ -118,16 +157,22 @@ int rows_per_cta(int i, int M, int R) {
 }
 
 // Opt instance i (mode) into the largest shared memory, once per device.
-cudaError_t ensure_zoom_smem(int i, int mode) {
-    static std::atomic<unsigned> done[kZoomInstances][3];
+cudaError_t ensure_smem(const void *kernel, std::atomic<unsigned> *done) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    std::atomic<unsigned> &d = done[i][mode];
-    if (dev < 32 && (d.load(std::memory_order_acquire) & (1u << dev))) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel_of(i, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    if (e == cudaSuccess && dev < 32) d.fetch_or(1u << dev, std::memory_order_acq_rel);
+    if (dev < 32 && (done->load(std::memory_order_acquire) & (1u << dev))) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess && dev < 32) done->fetch_or(1u << dev, std::memory_order_acq_rel);
     return e;
+}
+cudaError_t ensure_zoom_smem(int i, int mode) {
+    static std::atomic<unsigned> done[kZoomInstances][3];
+    return ensure_smem(kernel_of(i, mode), &done[i][mode]);
+}
+cudaError_t ensure_wide_smem(int i, int mode) {
+    static std::atomic<unsigned> done[kWideRest][2];
+    return ensure_smem(wide_kernel_of(i, mode), &done[i][mode]);
 }
 
 // Cost of one row (ps) on instance i by columns.  A run of R outputs starts at
@@ -161,51 +206,79 @@ double whole_cost(int i, const ZoomShape &z) {
     return (double)z.M * inst(i).cost * f;
 }
 
+// Cost of one row (ps) with first radix i and remaining length j of
+// zoom_wide.cuh.
+double wide_cost(int i, int j, const ZoomShape &z) {
+    const WideInst &w = wide_rest(j);
+    const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i);
+    double f = Rp % 8 == 0 && z.n_out % 8 == 0 ? 1.0 : Rp % 4 == 0 && z.n_out % 4 == 0 ? 1.2 : 1.5;
+    if (z.sub != 1) f *= 1.4;
+    const double pad = (double)((Rp + w.P - 1) / w.P * w.P) / Rp;
+    const double first = 1.1 + 0.02 * QA;
+    double rest = 2.2 + ((w.QB % 5 == 0 || w.QB % 7 == 0 || w.QB % 3 == 0) ? 0.15 : 0.0) +
+                  ((w.QC % 5 == 0 || w.QC % 7 == 0 || w.QC % 3 == 0) ? 0.15 : 0.0) + (w.P < 16 ? 0.3 : 0.0);
+    return (double)z.M * (first + rest * f * pad);
+}
+
+constexpr int kWideCode = 1 << 20;  // candidate codes of zoom_select: + 1024 i + j
+
 }  // namespace
 
-int zoom_class_L(const ZoomClass &c, int M) { return M / inst(c.inst).Q * inst(c.inst).QA; }
+int zoom_class_L(const ZoomClass &c, int M) {
+    if (c.wide >= 0) return M / (wide_rest(c.inst).QB * wide_rest(c.inst).QC);
+    return M / inst(c.inst).Q * inst(c.inst).QA;
+}
 
 void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomClass> *classes,
                  std::vector<int4> *list, std::vector<int> *rest) {
     classes->clear();
     list->clear();
     rest->clear();
-    // candidates: 2 i by columns, 2 i + 1 by whole rows; kRest the whole-row FFT kernels
+    // candidates: 2 i by columns, 2 i + 1 by whole rows, kWideCode + ... in two
+    // kernels, kRest the whole-row FFT kernels; each with its cost of a row and
+    // the widest band it takes wherever that starts
     constexpr int kRest = -1;
-    std::vector<int> open{kRest};
+    struct Cand {
+        int code;
+        double cost;
+        int cap;
+    };
+    std::vector<Cand> all{{kRest, z.rest_cost, 1 << 30}};
     for (int i = 0; i < kZoomInstances; ++i) {
         if (z.M % inst(i).Q != 0) continue;
-        const int R = z.M / inst(i).Q;
+        const int R = z.M / inst(i).Q, cap = inst(i).Q - (inst(i).NB - 1);  // the window starts at a multiple of NB
         // few residues leave a row's band product little use and its stores short
-        if (!z.rows_only && (R >= 4 || inst(i).P <= 4) && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem) open.push_back(2 * i);
+        if (!z.rows_only && (R >= 4 || inst(i).P <= 4) && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem)
+            all.push_back({2 * i, column_cost(i, z, S), cap});
         if (!z.phase && R >= 2 && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
             row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(i, rows_per_cta(i, z.M, R), R), R) <= kMaxSmem)
-            open.push_back(2 * i + 1);
+            all.push_back({2 * i + 1, whole_cost(i, z), cap});
     }
-    auto cost = [&](int k, int s) -> double {
-        if (k == kRest) return z.rest_cost;
-        const int i = k >> 1;
-        // the window starts at a multiple of NB
-        if (band[2 * s + 1] + band[2 * s] % inst(i).NB > inst(i).Q) return 1e30;
-        return (k & 1) ? whole_cost(i, z) : column_cost(i, z, S);
-    };
+    if (z.wide)
+        for (int j = 0; j < kWideRest; ++j) {
+            const int Qp = wide_rest(j).QB * wide_rest(j).QC;
+            if (z.M % Qp != 0) continue;
+            for (int i = 0; i < kWideFirst; ++i)
+                if ((z.M / Qp) % wide_radix(i) == 0 && z.M / Qp / wide_radix(i) <= kWideThreads)
+                    all.push_back({kWideCode + 1024 * i + j, wide_cost(i, j, z), wide_radix(i) * Qp});
+        }
+    std::stable_sort(all.begin(), all.end(), [](const Cand &a, const Cand &b) { return a.cost < b.cost; });
+    std::vector<Cand> open;  // those wider than every cheaper one, cheapest first
+    for (const Cand &c : all)
+        if (open.empty() || c.cap > open.back().cap) open.push_back(c);
     // every scale on its cheapest transform, then classes dissolved into the
     // remaining ones while the launch they save (3 us) outweighs the dearer
     // transforms of their scales, at a nominal number of channels
-    auto assign = [&](const std::vector<int> &o, std::vector<int> *to) -> double {
+    auto assign = [&](const std::vector<Cand> &o, std::vector<int> *to) -> double {
         double total = 0;
         std::vector<char> used(o.size(), 0);
         for (int s = 0; s < S; ++s) {
-            size_t b = o.size();
-            double c = 1e30;
-            for (size_t k = 0; k < o.size(); ++k) {
-                const double ck = cost(o[k], s);
-                if (ck < c) c = ck, b = k;
-            }
-            if (b == o.size()) return 1e300;
-            total += z.channels * c;
-            used[b] = 1;
-            if (to) (*to)[(size_t)s] = o[b];
+            size_t k = 0;
+            while (k < o.size() && o[k].cap < band[2 * s + 1]) ++k;
+            if (k == o.size()) return 1e300;
+            total += z.channels * o[k].cost;
+            used[k] = 1;
+            if (to) (*to)[(size_t)s] = o[k].code;
         }
         for (char u : used) total += u ? 3e6 : 0.0;
         return total;
@@ -213,16 +286,16 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
     std::vector<int> to((size_t)S, kRest);
     double total = assign(open, &to);
     {
-        std::vector<int> u;
-        for (int k : open)
-            if (std::find(to.begin(), to.end(), k) != to.end()) u.push_back(k);
+        std::vector<Cand> u;
+        for (const Cand &c : open)
+            if (std::find(to.begin(), to.end(), c.code) != to.end()) u.push_back(c);
         open = u;
     }
     while (open.size() > 1) {
         double best = total;
         size_t drop = open.size();
         for (size_t k = 0; k < open.size(); ++k) {
-            std::vector<int> o = open;
+            std::vector<Cand> o = open;
             o.erase(o.begin() + (long)k);
             const double t = assign(o, nullptr);
             if (t < best) best = t, drop = k;
@@ -231,19 +304,24 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
         open.erase(open.begin() + (long)drop);
         total = assign(open, &to);
     }
-    for (int k : open) {
+    for (const Cand &cand : open) {
+        const int k = cand.code;
         if (k == kRest) continue;
-        const int i = k >> 1, first = (int)list->size();
+        const bool wide = k >= kWideCode;
+        const int i = wide ? k & 1023 : k >> 1, first = (int)list->size(), nb = wide ? 1 : inst(i).NB;
         for (int s = 0; s < S; ++s)
             if (to[(size_t)s] == k)
-                list->push_back(make_int4(s, band[2 * s], band[2 * s + 1], band[2 * s] / inst(i).NB * inst(i).NB));
-        if ((int)list->size() > first) classes->push_back({i, first, (int)list->size() - first, (k & 1) != 0});
+                list->push_back(make_int4(s, band[2 * s], band[2 * s + 1], band[2 * s] / nb * nb));
+        if ((int)list->size() > first)
+            classes->push_back({i, first, (int)list->size() - first, !wide && (k & 1) != 0,
+                                wide ? (k - kWideCode) >> 10 : -1});
     }
     for (int s = 0; s < S; ++s)
         if (to[(size_t)s] == kRest) rest->push_back(s);
-    // the largest class first: the last launch's tail is then short
-    std::stable_sort(classes->begin(), classes->end(),
-                     [](const ZoomClass &a, const ZoomClass &b) { return a.ns > b.ns; });
+    // wide classes, then the largest first: the last launch's tail is short
+    std::stable_sort(classes->begin(), classes->end(), [](const ZoomClass &a, const ZoomClass &b) {
+        return (a.wide >= 0) != (b.wide >= 0) ? a.wide >= 0 : a.ns > b.ns;
+    });
 }
 
 cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const float2 *twl, const int4 *d_list,
@@ -295,7 +373,65 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     return cudaLaunchKernelExC(&cfg, kernel_of(c.inst, mode), params);
 }
 
+cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chans, const float2 *twl,
+                        const int4 *d_list, float2 *Z, int z_rows, cudaStream_t st) {
+    const WideInst &t = wide_rest(c.inst);
+    const int QA = wide_radix(c.wide);
+    WideArgs w;
+    w.z = args;
+    ZoomArgs &a = w.z;
+    const long long rows = chans * c.ns;
+    w.Z = Z;
+    w.Qp = t.QB * t.QC;
+    a.L = a.M / w.Qp;
+    a.R = a.L / QA;
+    a.twl = twl;
+    a.list = d_list + c.first;
+    a.ns = c.ns;
+    a.magM = zoom_magic((unsigned)a.M);
+    a.magSub = zoom_magic((unsigned)a.sub);
+    a.magL = zoom_magic((unsigned)a.L);
+    a.magR = zoom_magic((unsigned)a.R);
+    a.magNs = zoom_magic((unsigned)c.ns);
+    const int mode = a.oph || a.sub != 1 ? 1 : 0;
+    cudaError_t e = ensure_wide_smem(c.inst, mode);
+    if (e != cudaSuccess) return e;
+    // positions per CTA of the first kernel: about 512 butterflies
+    const int bb = std::max(4, std::min({w.Qp, 512 / a.R, (48 * 1024 / 8 - (QA + 1) * a.R) / QA}));
+    const int smem1 = (QA * bb + (QA + 1) * a.R) * (int)sizeof(float2);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    for (long long r0 = 0; r0 < rows && e == cudaSuccess; r0 += z_rows) {
+        w.row0 = (int)r0;
+        w.nrows = (int)std::min<long long>(z_rows, rows - r0);
+        void *params[] = {&w};
+        w.bb = bb;
+        w.groups = (w.Qp + bb - 1) / bb;
+        w.magG = zoom_magic((unsigned)w.groups);
+        cfg.gridDim = dim3((unsigned)(w.nrows * w.groups));
+        cfg.blockDim = dim3(kWideThreads);
+        cfg.dynamicSmemBytes = (size_t)smem1;
+        e = cudaLaunchKernelExC(&cfg, wide_first_entry(c.wide), params);
+        if (e != cudaSuccess) return e;
+        w.groups = (a.L + t.P - 1) / t.P;
+        w.magG = zoom_magic((unsigned)w.groups);
+        cfg.gridDim = dim3((unsigned)(w.nrows * w.groups));
+        cfg.blockDim = dim3((unsigned)t.T);
+        cfg.dynamicSmemBytes = (size_t)t.smem;
+        e = cudaLaunchKernelExC(&cfg, wide_kernel_of(c.inst, mode), params);
+    }
+    return e;
+}
+
 namespace {
+
+// Workspace of zoom_wide.cuh: rows whose Z stays in the 126 MB of L2.
+constexpr size_t kWideBytes = (size_t)64 << 20;
 
 // Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
 // with kernels compiled at its creation takes the same split of its scales).
@@ -313,6 +449,8 @@ struct ZoomPlan {
     std::vector<const float2 *> twl;  // per class: w_L^i, L = QA R
     int4 *d_list = nullptr;
     float2 *d_twl = nullptr;  // smooth lengths: those tables
+    float2 *d_wide = nullptr;  // the wide classes' workspace, wide_rows rows of M points
+    int wide_rows = 0;
     int M = 0, sub = 1, tws = 1;
     const float2 *tw = nullptr;
 };
@@ -321,6 +459,7 @@ void free_zoom_plan(ZoomPlan *z) {
     if (!z) return;
     cudaFree(z->d_list);
     cudaFree(z->d_twl);
+    cudaFree(z->d_wide);
     delete z;
 }
 
@@ -342,13 +481,14 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     sh.rest_cost = row_cost(p);
     sh.phase = (p->outputs & CWT_OUT_PHASE) != 0;
     sh.rows_only = false;
+    sh.wide = true;
     sh.channels = 64;
     sh.row_bytes = (double)p->n_out * (((p->outputs & CWT_OUT_COMPLEX) ? 8 : 0) + ((p->outputs & CWT_OUT_POWER) ? 4 : 0) +
                                        ((p->outputs & CWT_OUT_PHASE) ? 4 : 0));
     zoom_select(sh, S, band.data(), &classes, &list, &rest);
     // columns and grids stay within 31 bits
     for (const ZoomClass &c : classes)
-        if ((double)p->C * c.ns * (M / inst(c.inst).Q) >= 2147483647.0) list.clear();
+        if ((double)p->C * c.ns * (c.wide >= 0 ? 1 : M / inst(c.inst).Q) >= 2147483647.0) list.clear();
     if (list.empty()) return cudaSuccess;
     ZoomPlan *z = new ZoomPlan;
     p->zoom = z;  // freed with the plan, also on failure
@@ -370,6 +510,12 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
         z->twl.push_back(p->mr ? z->d_twl + at : twiddles_pow2(p->tw, L));
         at += (size_t)L;
     }
+    long long wide_rows = 0;
+    for (const ZoomClass &c : classes)
+        if (c.wide >= 0) wide_rows = std::max(wide_rows, (long long)p->C * c.ns);
+    wide_rows = std::min(wide_rows, (long long)std::max<size_t>(1, kWideBytes / (sizeof(float2) * (size_t)M)));
+    z->wide_rows = (int)wide_rows;
+    if (e == cudaSuccess && wide_rows) e = dmalloc(&z->d_wide, sizeof(float2) * (size_t)M * (size_t)wide_rows);
     if (e == cudaSuccess && !rest.empty()) {
         e = dmalloc(&p->rest_list, sizeof(int) * rest.size());
         if (e == cudaSuccess)
@@ -377,7 +523,8 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     p->rest_scales = (int)rest.size();
-    p->bytes += sizeof(int4) * list.size() + sizeof(int) * rest.size() + (p->mr ? sizeof(float2) * total_l : 0);
+    p->bytes += sizeof(int4) * list.size() + sizeof(int) * rest.size() + (p->mr ? sizeof(float2) * total_l : 0) +
+                sizeof(float2) * (size_t)M * (size_t)wide_rows;
     return e;
 }
 
@@ -417,7 +564,9 @@ cudaError_t launch_scale_block_zoom(const cwt_plan_s *p, float2 *out_c, float *o
     for (size_t k = 0; k < z->classes.size(); ++k) {
         a.after = after;
         after = true;
-        const cudaError_t e = zoom_launch(z->classes[k], a, p->C, z->twl[k], z->d_list, st);
+        const ZoomClass &c = z->classes[k];
+        const cudaError_t e = c.wide >= 0 ? wide_launch(c, a, p->C, z->twl[k], z->d_list, z->d_wide, z->wide_rows, st)
+                                          : zoom_launch(c, a, p->C, z->twl[k], z->d_list, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

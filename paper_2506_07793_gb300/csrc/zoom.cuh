@@ -186,7 +186,36 @@ __device__ __forceinline__ void zoom_store(T *dst, int step, int left, const flo
     }
 }
 
-// MODE 0: complex and power at every sample; 1: also phase and sub > 1.
+// The outputs t0 + step m < n_keep of one last-pass butterfly, MODE 0: complex
+// and power at every sample; 1: also phase and sub > 1.
+template <int L, int MODE>
+__device__ __forceinline__ void zoom_emit(const ZoomArgs &a, size_t obase, int t0, int step, int n_keep,
+                                          const float2 *v) {
+    if constexpr (MODE == 0) {
+        const int left = t0 + (L - 1) * step < n_keep ? L : (n_keep - t0 + step - 1) / step;
+        if (a.oc) zoom_store<L>(a.oc + obase + t0, step, left, v, [](float2 x) { return x; });
+        if (a.op)
+            zoom_store<L>(a.op + obase + t0, step, left, v,
+                          [](float2 x) { return fmaf(x.x, x.x, x.y * x.y); });
+    } else {
+#pragma unroll
+        for (int m = 0; m < L; ++m) {
+            const int t = t0 + m * step;
+            if (t >= n_keep) continue;
+            int o = t;
+            if (a.sub != 1) {
+                int rem;
+                zoom_divmod((unsigned)t, (unsigned)a.sub, a.magSub, o, rem);
+                if (rem != 0) continue;
+            }
+            if (a.oc) __stcs(a.oc + obase + o, v[m]);
+            if (a.op) __stcs(a.op + obase + o, fmaf(v[m].x, v[m].x, v[m].y * v[m].y));
+            if (a.oph) __stcs(a.oph + obase + o, phase_atan2(v[m].y, v[m].x));
+        }
+    }
+}
+
+// MODE as zoom_emit's.
 template <class Z, int MODE>
 __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_kernel(const ZoomArgs a) {
     constexpr int QA = Z::QA, QB = Z::QB, QC = Z::QC, P = Z::P, T = Z::T, QP = Z::QP, Q = Z::Q, QAP = Z::QAP;
@@ -327,28 +356,7 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_kernel(const ZoomArgs a) {
         for (int b = 0; b < LAST; ++b) v[b] = *CWT_SMEM(&x[b * (QAP * P)]);
         zoom_twiddle<LAST>(v, w, w8);
         dft_r<LAST, +1>(v);
-        if constexpr (MODE == 0) {
-            const int left = t0 + (LAST - 1) * step < n_keep ? LAST : (n_keep - t0 + step - 1) / step;
-            if (a.oc) zoom_store<LAST>(a.oc + obase + t0, step, left, v, [](float2 x) { return x; });
-            if (a.op)
-                zoom_store<LAST>(a.op + obase + t0, step, left, v,
-                                 [](float2 x) { return fmaf(x.x, x.x, x.y * x.y); });
-        } else {
-#pragma unroll
-            for (int m = 0; m < LAST; ++m) {
-                const int t = t0 + m * step;
-                if (t >= n_keep) continue;
-                int o = t;
-                if (a.sub != 1) {
-                    int rem;
-                    zoom_divmod((unsigned)t, (unsigned)a.sub, a.magSub, o, rem);
-                    if (rem != 0) continue;
-                }
-                if (a.oc) __stcs(a.oc + obase + o, v[m]);
-                if (a.op) __stcs(a.op + obase + o, fmaf(v[m].x, v[m].x, v[m].y * v[m].y));
-                if (a.oph) __stcs(a.oph + obase + o, phase_atan2(v[m].y, v[m].x));
-            }
-        }
+        zoom_emit<LAST, MODE>(a, obase, t0, step, n_keep, v);
     }
     if (a.after) griddep_wait();  // complete in stream order
 }

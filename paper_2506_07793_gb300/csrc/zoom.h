@@ -9,6 +9,8 @@
 
 #include "zoom.cuh"
 #include "zoom_list.h"
+#include "zoom_wide.cuh"
+#include "zoom_wide_list.h"
 
 namespace cwtk {
 
@@ -26,11 +28,25 @@ const void *zoom_entry(int mode);
                            : (const void *)&zoom_row_kernel<Z>;                 \
     }
 
-// Scales [first, first + ns) of a device list on one instance; rows: by
-// zoom_row_kernel.
+// The kernels of zoom_wide.cuh: first radix i, remaining length I in MODE 0 or 1.
+const void *wide_first_entry(int i);
+template <int I>
+const void *wide_rest_entry(int mode);
+
+#define CWT_WIDE_DEFINE(I, QB, QC, P, T, MINB)                                                          \
+    template <>                                                                                         \
+    const void *wide_rest_entry<I>(int mode) {                                                          \
+        using Z = WideCfg<QB, QC, P, T, MINB>;                                                          \
+        return mode == 0 ? (const void *)&wide_rest_kernel<Z, 0> : (const void *)&wide_rest_kernel<Z, 1>; \
+    }
+
+// Scales [first, first + ns) of a device list on one instance of zoom_kernel, of
+// zoom_row_kernel (rows), or on first radix `wide` and remaining length `inst`
+// of zoom_wide.cuh.
 struct ZoomClass {
     int inst, first, ns;
     bool rows;
+    int wide;  // -1: not wide
 };
 
 // What zoom_select decides from: a row of N bins on M points of which every
@@ -40,7 +56,7 @@ struct ZoomClass {
 struct ZoomShape {
     int N, M, sub, n_out;
     double rest_cost;
-    bool phase, rows_only;
+    bool phase, rows_only, wide;  // only zoom_row_kernel; zoom_wide.cuh allowed
     double channels;   // nominal, for the cost of a launch against that of its rows
     double row_bytes;  // output bytes of one row
 };
@@ -54,5 +70,8 @@ int zoom_class_L(const ZoomClass &c, int M);  // points of its first pass's tabl
 // n_out, sub, n_keep, after and the batch's fields.
 cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const float2 *twl, const int4 *d_list,
                         cudaStream_t st);
+// Launch wide class c with a workspace of z_rows rows of M points.
+cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &a, long long chans, const float2 *twl, const int4 *d_list,
+                        float2 *Z, int z_rows, cudaStream_t st);
 
 }  // namespace cwtk

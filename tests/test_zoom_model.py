@@ -82,3 +82,41 @@ def test_columns_equal_the_plain_inverse_dft(QA, QB, QC, P, M, fold):
             got.update(zoom_columns(Y, b0, M, N, QA, QB, QC, P, list(range(r0, min(R, r0 + P)))))
         assert sorted(got) == list(range(M))
         np.testing.assert_allclose([got[t] for t in range(M)], ref, rtol=0, atol=1e-11 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("QA,QB,QC,M,fold", [(2, 4, 5, 240, 1), (5, 4, 4, 320, 2), (8, 4, 8, 1024, 1), (9, 5, 7, 945, 1)])
+def test_two_kernel_form_equals_the_plain_inverse_dft(QA, QB, QC, M, fold):
+    """csrc/zoom_wide.cuh: the first kernel's Z[b][t'] and the second's passes."""
+    rng = np.random.default_rng(M + QA)
+    Qp, N = QB * QC, M * fold
+    Q, Rp = QA * Qp, M // Qp
+    R = Rp // QA
+    for B, b0 in [(1, 0), (Q, N - 2), (Q - 1, N - Q // 2), (Q // 2, 3), (Q, Qp - 1)]:
+        Y = rng.standard_normal(B) + 1j * rng.standard_normal(B)
+        Z = np.full((Qp, Rp), np.nan, complex)
+        for b in range(Qp):
+            y, g = np.zeros(QA, complex), np.zeros(QA, int)
+            for p in range(QA):
+                k = b + Qp * p - b0 % Q
+                k += Q + b0 if k < 0 else b0          # the bin of the window [b0, b0 + Q)
+                y[p] = Y[k - b0] if k - b0 < B else 0.0
+                base = b0 // Qp + (1 if b < b0 % Qp else 0)
+                g[p] = (p - base) % QA + base
+                assert k == b + Qp * g[p]
+            for r in range(R):
+                v = np.fft.ifft(y * w(Rp, g * r)) * QA
+                Z[b, r + R * np.arange(QA)] = v
+        out = np.full(M, np.nan, complex)
+        for t1 in range(Rp):
+            tile = np.full(Qp, np.nan, complex)
+            for b1 in range(QC):
+                b2 = np.arange(QB)
+                assert QC * t1 < M
+                tile[b1 + QC * b2] = np.fft.ifft(Z[b1 + QC * b2, t1] * w(M, QC * t1) ** b2) * QB
+            for k2 in range(QB):
+                t0 = t1 + Rp * k2
+                v = np.fft.ifft(tile[QC * k2 + np.arange(QC)] * w(M, t0) ** np.arange(QC)) * QC
+                out[t0 + Rp * QB * np.arange(QC)] = v
+        k = b0 + np.arange(B)
+        ref = np.exp(2j * np.pi * np.outer(np.arange(M), k % M) / M) @ Y
+        np.testing.assert_allclose(out, ref, rtol=0, atol=1e-11 * np.abs(ref).max())
