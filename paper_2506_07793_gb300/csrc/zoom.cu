@@ -374,14 +374,13 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
 }
 
 cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chans, const float2 *twl,
-                        const int4 *d_list, float2 *Z, int z_rows, cudaStream_t st) {
+                        const int4 *d_list, float2 *Z, int z_rows, int *turn, cudaStream_t st) {
     const WideInst &t = wide_rest(c.inst);
     const int QA = wide_radix(c.wide);
     WideArgs w;
     w.z = args;
     ZoomArgs &a = w.z;
     const long long rows = chans * c.ns;
-    w.Z = Z;
     w.Qp = t.QB * t.QC;
     a.L = a.M / w.Qp;
     a.R = a.L / QA;
@@ -408,6 +407,8 @@ cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chan
     cfg.numAttrs = 1;
     for (long long r0 = 0; r0 < rows && e == cudaSuccess; r0 += z_rows) {
         w.row0 = (int)r0;
+        w.Z = Z + (size_t)(*turn & 1) * (size_t)z_rows * (size_t)a.M;
+        ++*turn;
         w.nrows = (int)std::min<long long>(z_rows, rows - r0);
         void *params[] = {&w};
         w.bb = bb;
@@ -424,14 +425,15 @@ cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chan
         cfg.blockDim = dim3((unsigned)t.T);
         cfg.dynamicSmemBytes = (size_t)t.smem;
         e = cudaLaunchKernelExC(&cfg, wide_kernel_of(c.inst, mode), params);
+        a.after = 1;
     }
     return e;
 }
 
 namespace {
 
-// Workspace of zoom_wide.cuh: rows whose Z stays in the 126 MB of L2.
-constexpr size_t kWideBytes = (size_t)64 << 20;
+// Half the workspace of zoom_wide.cuh: rows whose Z stays in the 126 MB of L2.
+constexpr size_t kWideBytes = (size_t)40 << 20;
 
 // Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
 // with kernels compiled at its creation takes the same split of its scales).
@@ -449,7 +451,7 @@ struct ZoomPlan {
     std::vector<const float2 *> twl;  // per class: w_L^i, L = QA R
     int4 *d_list = nullptr;
     float2 *d_twl = nullptr;  // smooth lengths: those tables
-    float2 *d_wide = nullptr;  // the wide classes' workspace, wide_rows rows of M points
+    float2 *d_wide = nullptr;  // the wide classes' workspace, twice wide_rows rows of M points
     int wide_rows = 0;
     int M = 0, sub = 1, tws = 1;
     const float2 *tw = nullptr;
@@ -515,7 +517,7 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
         if (c.wide >= 0) wide_rows = std::max(wide_rows, (long long)p->C * c.ns);
     wide_rows = std::min(wide_rows, (long long)std::max<size_t>(1, kWideBytes / (sizeof(float2) * (size_t)M)));
     z->wide_rows = (int)wide_rows;
-    if (e == cudaSuccess && wide_rows) e = dmalloc(&z->d_wide, sizeof(float2) * (size_t)M * (size_t)wide_rows);
+    if (e == cudaSuccess && wide_rows) e = dmalloc(&z->d_wide, 2 * sizeof(float2) * (size_t)M * (size_t)wide_rows);
     if (e == cudaSuccess && !rest.empty()) {
         e = dmalloc(&p->rest_list, sizeof(int) * rest.size());
         if (e == cudaSuccess)
@@ -524,7 +526,7 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     p->rest_scales = (int)rest.size();
     p->bytes += sizeof(int4) * list.size() + sizeof(int) * rest.size() + (p->mr ? sizeof(float2) * total_l : 0) +
-                sizeof(float2) * (size_t)M * (size_t)wide_rows;
+                2 * sizeof(float2) * (size_t)M * (size_t)wide_rows;
     return e;
 }
 
@@ -560,12 +562,14 @@ cudaError_t launch_scale_block_zoom(const cwt_plan_s *p, float2 *out_c, float *o
     // forward FFTs waits for them before it reads a spectrum; a later one may
     // start when every CTA of the one before has passed that point, reads the
     // spectra at once and waits at its end, so that the stream's order holds.
+    int turn = 0;  // the workspace's halves
     bool after = p->rest_scales > 0;  // the whole-row kernel before saw the forward FFTs complete
     for (size_t k = 0; k < z->classes.size(); ++k) {
         a.after = after;
         after = true;
         const ZoomClass &c = z->classes[k];
-        const cudaError_t e = c.wide >= 0 ? wide_launch(c, a, p->C, z->twl[k], z->d_list, z->d_wide, z->wide_rows, st)
+        const cudaError_t e = c.wide >= 0 ? wide_launch(c, a, p->C, z->twl[k], z->d_list, z->d_wide, z->wide_rows,
+                                                        &turn, st)
                                           : zoom_launch(c, a, p->C, z->twl[k], z->d_list, st);
         if (e != cudaSuccess) return e;
     }

@@ -358,7 +358,8 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_kernel(const ZoomArgs a) {
         dft_r<LAST, +1>(v);
         zoom_emit<LAST, MODE>(a, obase, t0, step, n_keep, v);
     }
-    if (a.after) griddep_wait();  // complete in stream order
+    // complete in stream order: one CTA outlives the kernel before
+    if (a.after && blockIdx.x == gridDim.x - 1) griddep_wait();
 }
 
 // Whole rows of M <= kZoomRowPoints points: a CTA holds all R residues of nr
@@ -556,7 +557,8 @@ __global__ void __launch_bounds__(Z::T, Z::MINB) zoom_row_kernel(const ZoomArgs 
             zoom_store<LAST>(a.op + z.base + t0, step, left, v,
                              [](float2 x) { return fmaf(x.x, x.x, x.y * x.y); });
     }
-    if (a.after) griddep_wait();  // complete in stream order
+    // complete in stream order: one CTA outlives the kernel before
+    if (a.after && blockIdx.x == gridDim.x - 1) griddep_wait();
 }
 
 }  // namespace cwtk

@@ -70,8 +70,9 @@ int zoom_class_L(const ZoomClass &c, int M);  // points of its first pass's tabl
 // n_out, sub, n_keep, after and the batch's fields.
 cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const float2 *twl, const int4 *d_list,
                         cudaStream_t st);
-// Launch wide class c with a workspace of z_rows rows of M points.
+// Launch wide class c with a workspace of two halves of z_rows rows of M
+// points, used by turns (*turn counts on from class to class).
 cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &a, long long chans, const float2 *twl, const int4 *d_list,
-                        float2 *Z, int z_rows, cudaStream_t st);
+                        float2 *Z, int z_rows, int *turn, cudaStream_t st);
 
 }  // namespace cwtk

@@ -14,7 +14,10 @@
 //                      consecutive t' per CTA, two passes Q' = QB QC over a
 //                      tile in shared memory, stores as zoom_kernel's.
 // Z takes 8 bytes per output each way.  The host runs the rows in chunks whose
-// Z stays in L2 (zoom.cu).  Bound by instruction issue like zoom_kernel.
+// Z stays in L2 (zoom.cu), in two halves of the workspace by turns: the first
+// kernel of a chunk starts as the second of the chunk before it runs out of
+// CTAs to launch (each waits, as programmatic dependents, only for what it
+// needs).  Bound by instruction issue like zoom_kernel.
 #pragma once
 
 #include "zoom.cuh"
@@ -58,7 +61,9 @@ __global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 3) wide_first_ker
             if (i >= (unsigned)Rp) i -= (unsigned)Rp;
         }
     }
-    griddep_wait();  // the spectra, and the last reads of Z
+    // The spectra are complete when a.after.  This half of Z is free: the kernel
+    // before has passed its wait for a kernel that outlived its last reader.
+    if (!a.after) griddep_wait();
     griddep_launch();
     const int b0 = grp * bb, nb = min(bb, Qp - b0), wm = sc.w % Q;
     const float2 *X = a.spec + (size_t)c * N;
@@ -78,6 +83,8 @@ __global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 3) wide_first_ker
         *CWT_SMEM(&Y[i]) = y;
     }
     __syncthreads();
+    // one CTA outlives the second kernel of the chunk before
+    if (a.after && blockIdx.x == gridDim.x - 1) griddep_wait();
     if (th >= TP) return;
     float2 e[QA];
 #pragma unroll
