@@ -207,16 +207,18 @@ double whole_cost(int i, const ZoomShape &z) {
 }
 
 // Cost of one row (ps) with first radix i and remaining length j of
-// zoom_wide.cuh.
+// zoom_wide.cuh (mean of power only and complex and power, launch by launch
+// over 38 rows of 131072 points less the launches' ends: first kernel 1.4 ps
+// per point, second 8 x 32 2.1, 16 x 32 2.4).
 double wide_cost(int i, int j, const ZoomShape &z) {
     const WideInst &w = wide_rest(j);
     const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i);
     double f = Rp % 8 == 0 && z.n_out % 8 == 0 ? 1.0 : Rp % 4 == 0 && z.n_out % 4 == 0 ? 1.2 : 1.5;
     if (z.sub != 1) f *= 1.4;
     const double pad = (double)((Rp + w.P - 1) / w.P * w.P) / Rp;
-    const double first = 1.1 + 0.02 * QA;
-    double rest = 2.2 + ((w.QB % 5 == 0 || w.QB % 7 == 0 || w.QB % 3 == 0) ? 0.15 : 0.0) +
-                  ((w.QC % 5 == 0 || w.QC % 7 == 0 || w.QC % 3 == 0) ? 0.15 : 0.0) + (w.P < 16 ? 0.3 : 0.0);
+    const double first = QA <= 8 ? 1.4 : 1.4 + 0.025 * (QA - 8) + (QA > 16 ? 0.02 * (QA - 16) : 0.0);
+    const double rest = 1.95 + 0.0007 * (w.QB * w.QC) + ((w.QB % 5 == 0 || w.QB % 7 == 0 || w.QB % 3 == 0) ? 0.15 : 0.0) +
+                  ((w.QC % 5 == 0 || w.QC % 7 == 0 || w.QC % 3 == 0) ? 0.15 : 0.0)  + (w.P < 16 ? 0.1 : 0.0);
     return (double)z.M * (first + rest * f * pad);
 }
 
@@ -396,8 +398,9 @@ cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chan
     cudaError_t e = ensure_wide_smem(c.inst, mode);
     if (e != cudaSuccess) return e;
     // positions per CTA of the first kernel: about 512 butterflies
-    const int bb = std::max(4, std::min({w.Qp, 512 / a.R, (48 * 1024 / 8 - (QA + 1) * a.R) / QA}));
-    const int smem1 = (QA * bb + (QA + 1) * a.R) * (int)sizeof(float2);
+    const int et = QA <= 16 ? QA + 1 : 2 * QA;  // its table's rows
+    const int bb = std::max(4, std::min({w.Qp, 512 / a.R, (48 * 1024 / 8 - et * a.R) / QA}));
+    const int smem1 = (QA * bb + et * a.R) * (int)sizeof(float2);
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -432,16 +435,19 @@ cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chan
 
 namespace {
 
-// Half the workspace of zoom_wide.cuh: rows whose Z stays in the 126 MB of L2.
-constexpr size_t kWideBytes = (size_t)40 << 20;
+// Half the workspace of zoom_wide.cuh (32 x 122880 x 128 power: 1.80 ms with 28
+// MB, 1.69 with 40, 1.61 with 57, 1.67 with 80, 1.62 with 400).
+constexpr size_t kWideBytes = (size_t)56 << 20;
 
 // Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
 // with kernels compiled at its creation takes the same split of its scales).
 double row_cost(const cwt_plan_s *p) {
     if (p->precision != CWT_PREC_FP32) return (double)p->N * 10.0;  // tensor-core stages: 340 us per 1024 x 32768
-    if (!p->mr) return (double)p->M * (p->M <= kMaxFft ? 3.3 : 7.2);
+    // the rest are wide bands, whose first pass is dense: 64 x 10000, 20 of 100
+    // scales, complex and power: 5.6 ps per point at 16384, 4.4 at 10000
+    if (!p->mr) return (double)p->M * (p->M <= kMaxFft ? 4.4 : 7.4);
     if (p->cl > 1) return (double)p->N * (p->sch.fixed_cl >= 0 ? 7.2 : 30.0);
-    return (double)p->N * (p->sch.fixed >= 0 ? 3.4 : p->sch.fast >= 0 ? 6.0 : 14.0);
+    return (double)p->N * (p->sch.fixed >= 0 ? 4.1 : p->sch.fast >= 0 ? 6.5 : 14.0);
 }
 
 }  // namespace

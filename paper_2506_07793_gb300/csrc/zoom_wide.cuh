@@ -35,12 +35,15 @@ struct WideArgs {
 constexpr int kWideThreads = 128;
 
 template <int QA>
-__global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 3) wide_first_kernel(const WideArgs w) {
+__global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 4) wide_first_kernel(const WideArgs w) {
     constexpr int T = kWideThreads;
+    // up to 16 points the modulation stays in registers, above it takes them
+    // from the butterfly (QA = 32: 2.9 ps per point) and is read per use
+    constexpr bool kKeep = QA <= 16;
     extern __shared__ float2 wsm[];
     const ZoomArgs &a = w.z;
     const int R = a.R, N = a.N, Qp = w.Qp, Q = QA * Qp, Rp = a.L, bb = w.bb;
-    float2 *const Y = wsm, *const E = wsm + QA * bb;  // [QA][bb], [QA + 1][R]
+    float2 *const Y = wsm, *const E = wsm + QA * bb;  // [QA][bb]; [QA + 1][R], or [2][QA][R] for b from and below rho
     const int tid = (int)threadIdx.x;
     int lrow, grp, th, r, c, si;
     zoom_divmod(blockIdx.x, (unsigned)w.groups, w.magG, lrow, grp);
@@ -56,7 +59,13 @@ __global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 3) wide_first_ker
         for (int j = th; j <= QA; j += TP) {
             int p = pst + j;
             if (p >= QA) p -= QA;
-            *CWT_SMEM(&E[(j == QA ? QA : p) * R + r]) = __ldg(&a.twl[i]);
+            const float2 e = __ldg(&a.twl[i]);
+            if constexpr (kKeep) {
+                *CWT_SMEM(&E[(j == QA ? QA : p) * R + r]) = e;
+            } else {
+                if (j < QA) *CWT_SMEM(&E[p * R + r]) = e;
+                if (j > 0) *CWT_SMEM(&E[(QA + (j == QA ? pst : p)) * R + r]) = e;
+            }
             i += stride;
             if (i >= (unsigned)Rp) i -= (unsigned)Rp;
         }
@@ -86,27 +95,35 @@ __global__ void __launch_bounds__(kWideThreads, QA <= 16 ? 5 : 3) wide_first_ker
     // one CTA outlives the second kernel of the chunk before
     if (a.after && blockIdx.x == gridDim.x - 1) griddep_wait();
     if (th >= TP) return;
-    float2 e[QA];
+    float2 e[kKeep ? QA : 1], ex = make_float2(0.f, 0.f);
+    if constexpr (kKeep) {
 #pragma unroll
-    for (int p = 0; p < QA; ++p) e[p] = *CWT_SMEM(&E[p * R + r]);
-    float2 ex = *CWT_SMEM(&E[QA * R + r]);
+        for (int p = 0; p < QA; ++p) e[p] = *CWT_SMEM(&E[p * R + r]);
+        ex = *CWT_SMEM(&E[QA * R + r]);
+    }
     bool wrapped = false;
     float2 *out = w.Z + ((size_t)lrow * Qp + b0) * Rp + r;
 #pragma unroll 1
     for (int j = th; j < nb; j += TP) {
-        if ((b0 + j < rho) != wrapped) {
-            wrapped = !wrapped;
-            const float2 t = ex;
-#pragma unroll
-            for (int p = 0; p < QA; ++p)
-                if (p == pst) {
-                    ex = e[p];
-                    e[p] = t;
-                }
-        }
         float2 v[QA];
+        if constexpr (kKeep) {
+            if ((b0 + j < rho) != wrapped) {
+                wrapped = !wrapped;
+                const float2 t = ex;
 #pragma unroll
-        for (int p = 0; p < QA; ++p) v[p] = cmul(*CWT_SMEM(&Y[p * bb + j]), e[p]);
+                for (int p = 0; p < QA; ++p)
+                    if (p == pst) {
+                        ex = e[p];
+                        e[p] = t;
+                    }
+            }
+#pragma unroll
+            for (int p = 0; p < QA; ++p) v[p] = cmul(*CWT_SMEM(&Y[p * bb + j]), e[p]);
+        } else {
+            const float2 *ep = E + (b0 + j < rho ? QA * R : 0) + r;
+#pragma unroll
+            for (int p = 0; p < QA; ++p) v[p] = cmul(*CWT_SMEM(&Y[p * bb + j]), *CWT_SMEM(&ep[p * R]));
+        }
         dft_r<QA, +1>(v);
         float2 *o = out + (size_t)j * Rp;
 #pragma unroll
