@@ -1,34 +1,32 @@
-// batch.cu -- many epochs of uneven length in one persistent launch.
+// batch.cu -- many epochs of uneven length in one call.
 //
 // The paper loops over recordings in Python (Sections "Comparison between
 // devices and software" and "Wavelength and flexibility"); here a batch of
 // epochs, each with its own length n_e and hence its own padded length
 // N_e = next power of two >= max(n_e, 32) (Section "Fast Fourier transform"),
-// is one persistent kernel replayed from a CUDA graph.
+// is one launch per stage for all of them.
 //
-// Work item = (epoch, group of G channels) with G * N_e = one tile of kTile
-// points (G capped by the channel count).  Per item the CTA
+// The narrow-band scales (most or all: the band is 4 ... 36% of N_e / f on the
+// batching workload) run by residue classes, zoom_row_kernel of zoom.cuh, one
+// launch per padded length and class of scales over all its epochs.  They read
+// a window of bins, an eighth of the spectrum; the workspace that carries it is
+// kept below kWsBytes by taking the epochs in chunks.  Where every scale of a
+// padded length does so, its forward FFTs are batch_forward.cu's.
+//
+// Otherwise a persistent kernel, replayed from a CUDA graph, takes work items
+// of one epoch and G channels with G * N_e = one tile of kTile points (G capped
+// by the channel count), from an atomic counter, largest FFTs first.  Per item
+// the CTA
 //   1. runs the forward FFT of the G channels (Eq. 2, one FFT per channel)
 //      and keeps the spectra in shared memory -- they never reach HBM;
-//   2. stores the window of bins that the narrow-band scales of that length
-//      read (see below);
+//   2. stores the window of bins that the narrow-band scales read;
 //   3. for every (channel, scale) row of the other scales: band product with
 //      the FP64-generated bank of length N_e (Eq. 3), spectral fold by the
 //      power-of-two factor f of the decimation, inverse FFT of N_e / f points,
 //      crop / decimate / reduce and coalesced stores (Section "Precision").
-// CTAs pull items from an atomic counter, largest FFTs first.
-//
-// The narrow-band scales (most: the band is 4 ... 36% of N_e / f on the
-// batching workload) then run by residue classes, zoom_row_kernel of zoom.cuh,
-// one launch per padded length and class of scales over all its epochs.  Their
-// bins are an eighth of the spectrum; the workspace that carries them is kept
-// below kWsBytes by taking the epochs in chunks.
-//
-// The schedule is a rule: inverse rows on 16 points per thread (two CTAs per
-// SM; 47 ms per batch of 2048 epochs against 81 on 32 points), on 32 only for
-// batches with a row that 16 cannot stage, and items largest first (59 and
-// 131 ms in input order).  Timing the four on the first batch of every new
-// set of epoch lengths cost 14 batches' time.
+// Its rows take 16 points per thread (two CTAs per SM; 47 ms per batch of 2048
+// epochs against 81 on 32 points), 32 only in batches with a row that 16 cannot
+// stage, items largest first (59 and 131 ms in input order).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -197,7 +195,10 @@ cudaError_t make_length(cwt_plan_s *p, int L, cudaStream_t st, BatchLength *out)
         sh.M = l.M = N / f;
         sh.sub = p->d / f;
         sh.n_out = 0;  // epochs of any length
-        sh.rest_cost = 5.0 * batch_inverse_length(N, p->d);  // measured, 5.5 ps less the forward FFTs
+        // ps: a row here takes 4.2 ps per point, and the first one brings the forward FFTs
+        // of its length with it (7 of 64 scales of 8192-point rows: 6.3 ps per point in all,
+        // 4.4 on 32 x 32 by residue classes)
+        sh.rest_cost = 8.0 * batch_inverse_length(N, p->d);
         // rows subsampled past the fold (odd d) keep the kernel here: 0.92 against 0.99 ms
         // for 144 epochs of 8 channels at d = 5
         sh.phase = (p->outputs & CWT_OUT_PHASE) != 0 || sh.sub != 1;
@@ -260,7 +261,7 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
     std::vector<BatchItem> items;
     std::vector<ZoomEpoch> eps;
     std::vector<BatchChunk> chunks;
-    size_t ws_max = 0;
+    size_t ws_max = 0, n_items = 0;
     int max_m = 0;
     b->ready = false;
     for (int first = 0; first < n_epochs;) {
@@ -282,7 +283,8 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
                 const int N = 1 << L, n_out = (ep.samples + d - 1) / d, sub = d / std::gcd(N, d);
                 max_m = std::max(max_m, l.nrest ? batch_inverse_length(N, d) : 0);
                 const int G = std::max(1, std::min(C, kTile / N));
-                for (int c0 = 0; c0 < C; c0 += G) {
+                n_items += (size_t)((C + G - 1) / G);
+                for (int c0 = 0; l.nrest && c0 < C; c0 += G) {  // the others: batch_forward.cu
                     BatchItem it{};
                     it.in_off = ep.in_offset + (long long)c0 * ep.samples;
                     it.out_off = ep.out_offset + (long long)c0 * S * n_out;
@@ -292,7 +294,7 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
                     it.G = std::min(G, C - c0);
                     items.push_back(it);
                 }
-                eps.push_back({(long long)ws, ep.out_offset, n_out, sub * (n_out - 1) + 1});
+                eps.push_back({(long long)ws, ep.out_offset, ep.in_offset, n_out, sub * (n_out - 1) + 1, ep.samples, 0});
                 ws += (size_t)C * (size_t)l.wn;
             }
             ch.eps[L] = eps.size() - ch.ep0[L];
@@ -302,10 +304,10 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
         chunks.push_back(ch);
         first = last;
     }
-    cudaError_t e = grow(&b->d_items, &b->items_cap, items.size());
+    cudaError_t e = grow(&b->d_items, &b->items_cap, std::max<size_t>(items.size(), 1));
     if (e == cudaSuccess) e = grow(&b->d_eps, &b->eps_cap, eps.size());
     if (e == cudaSuccess) e = grow(&b->d_ws, &b->ws_cap, ws_max);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !items.empty())
         e = cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_eps, eps.data(), eps.size() * sizeof(ZoomEpoch), cudaMemcpyHostToDevice, st);
@@ -318,7 +320,7 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
     for (int i = 0; i < 4; ++i) b->tune_ms[i] = !ri16 && i % 2 == 0 ? -1.0 : 0.0;
     b->shape.assign(epochs, epochs + n_epochs);
     b->chunks = chunks;
-    b->n_items = items.size();
+    b->n_items = n_items;
     b->ready = true;
     return cudaSuccess;
 }
@@ -372,8 +374,23 @@ cudaError_t batch_run(cwt_plan_s *p, const float *in, float2 *oc, float *op, flo
         a.tw = p->tw;
         a.S = p->S;
         a.d = p->d;
-        e = batch_graph(b, b->ri, a, grid);
-        if (e == cudaSuccess) e = cudaGraphLaunch(b->exec, st);
+        if (ch.items) {
+            e = batch_graph(b, b->ri, a, grid);
+            if (e == cudaSuccess) e = cudaGraphLaunch(b->exec, st);
+        }
+        BatchForwardArgs f = {};
+        f.in = in;
+        f.ws = b->d_ws;
+        f.tw = p->tw;
+        f.C = p->C;
+        for (int L = 0; L <= kMaxBatchLog2; ++L) {
+            if (b->len[L].nrest || b->len[L].classes.empty()) continue;
+            f.eps[L] = b->d_eps + ch.ep0[L];
+            f.rows[L] = (int)ch.eps[L] * p->C;
+            f.w0[L] = b->len[L].w0;
+            f.wn[L] = b->len[L].wn;
+        }
+        if (e == cudaSuccess) e = launch_batch_forward(f, st);
         if (e != cudaSuccess) return e;
         b->grid = grid;
         ++b->launches;

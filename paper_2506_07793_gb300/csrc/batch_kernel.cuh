@@ -65,6 +65,19 @@ __host__ __device__ inline int batch_inverse_length(int N, int d) {
 // The kernel for RI = 16 or 32 (defined in batch_k16.cu / batch_k32.cu).
 const void *batch_kernel_ptr(int ri);
 
+// batch_forward.cu: per log2 N the epochs, their rows (epochs x channels) and
+// the window of bins; groups is filled by the launch.
+struct ZoomEpoch;
+struct BatchForwardArgs {
+    const float *in;
+    const ZoomEpoch *eps[kMaxBatchLog2 + 1];
+    int rows[kMaxBatchLog2 + 1], groups[kMaxBatchLog2 + 1], w0[kMaxBatchLog2 + 1], wn[kMaxBatchLog2 + 1];
+    float2 *ws;
+    const float2 *tw;
+    int C;
+};
+cudaError_t launch_batch_forward(BatchForwardArgs a, cudaStream_t st);
+
 #ifdef CWT_BATCH_KERNELS
 namespace {
 

@@ -33,8 +33,8 @@ namespace cwtk {
 
 // An epoch of a batch: element offsets of channel 0's spectrum and outputs.
 struct ZoomEpoch {
-    long long spec, out;
-    int n_out, n_keep;
+    long long spec, out, in;  // element offsets of channel 0: window of bins, output, input
+    int n_out, n_keep, n, pad;
 };
 
 struct ZoomArgs {
