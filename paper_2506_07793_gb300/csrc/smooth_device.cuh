@@ -40,8 +40,11 @@ __device__ __forceinline__ void mr_sb_row(const MrArgs &a, int N, int T, int R0,
     const int rr = rs.rr < rows ? rs.rr : 0;
     float2 *sm = mrsm + (size_t)rr * (N + (N >> 4));
     const int c = row / a.ns;
-    int s = row - c * a.ns;
-    if (a.list) s = a.list[s];
+    int s = row - c * a.ns, orow = row;
+    if (a.list) {
+        s = a.list[s];
+        orow = c * a.S + s;
+    }
     const float2 *X = a.spec + (size_t)c * N;
     const float *W = a.bank + (size_t)s * N;
     const int b0 = a.band[2 * s], B = a.band[2 * s + 1];
@@ -73,7 +76,7 @@ __device__ __forceinline__ void mr_sb_row(const MrArgs &a, int N, int T, int R0,
     if (!rs.active) return;
     // epilogue: crop to t < n, keep t = sub * o, write the requested outputs
     // (consecutive threads take consecutive o: coalesced stores)
-    const size_t obase = (size_t)(c * a.S + s) * (size_t)a.n_out;
+    const size_t obase = (size_t)orow * (size_t)a.n_out;
     const int sub = a.sub, n_out = a.n_out;
     if (a.f64) {
         double2 *oc = (double2 *)a.out_c + obase;

@@ -42,8 +42,12 @@ cudaError_t mr_sb_launch(const cwt_plan_s *p, const MrArgs &a, cudaStream_t st) 
     const int rows = mr_launch_rows(p->sch, a.total_rows);
     const int smem = rows * (p->N + (p->N >> 4)) * 8;
     const int threads = (rows * p->sch.T + 31) & ~31;
-    return launch_dependent(mr_scale_block_kernel<RA, RB>, (a.total_rows + rows - 1) / rows, threads, smem, st, a, p->sch,
-                            rows);
+    const int grid = (a.total_rows + rows - 1) / rows;
+    // Double rows start after the forward FFTs: 106 x 93 x 120 points take 26.6
+    // us, 28.7 overlapped; float rows overlap (26 x 113 x 1845: 49.2, 51.3).
+    if (!a.f64) return launch_dependent(mr_scale_block_kernel<RA, RB>, grid, threads, smem, st, a, p->sch, rows);
+    mr_scale_block_kernel<RA, RB><<<grid, threads, smem, st>>>(a, p->sch, rows);
+    return cudaGetLastError();
 }
 
 // Forward FFT of each zero-padded channel (float32 or float64 samples), Eq. 2;
