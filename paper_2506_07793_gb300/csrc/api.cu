@@ -586,7 +586,7 @@ cwt_status cwt_execute_batch(cwt_plan p, const cwt_epoch *epochs, int n_epochs, 
     if (wp && !device_ptr_ok(d_power, p->device)) return CWT_EINVAL;
     if (wph && !device_ptr_ok(d_phase, p->device)) return CWT_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    // prepare (banks, work items, autotuning on a new shape), then one timed launch
+    // prepare (banks, work items, workspace for a new shape), then the timed launches
     cudaError_t e = cwtk::batch_execute(p, epochs, n_epochs, (const float *)d_in, (float2 *)d_complex,
                                         (float *)d_power, (float *)d_phase, st, true);
     cwtk::ProfEvent ev{};

@@ -431,6 +431,11 @@ cudaError_t batch_run(cwt_plan_s *p, const float *in, float2 *oc, float *op, flo
 
 cudaError_t batch_execute(cwt_plan_s *p, const cwt_epoch *epochs, int n_epochs, const float *in,
                           float2 *oc, float *op, float *oph, cudaStream_t st, bool prepare_only) {
+    // A captured batch would replay into a workspace that a later shape replaces.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
     if (!prepare_only) return batch_run(p, in, oc, op, oph, st);
     try {
         return batch_prepare(p, epochs, n_epochs, st);

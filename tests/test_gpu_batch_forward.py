@@ -43,3 +43,27 @@ def test_batches_of_narrow_bands_match_the_oracle(case):
             assert power_err(got, ref).max() <= FP32_TOL, n
     finally:
         lib.cwt_plan_destroy(plan)
+
+
+def test_a_batch_inside_a_capture_is_refused():
+    import torch
+    import paper_2506_07793_gb300 as lib
+    o = lib.cwt_options_init()
+    o.decimation = 4
+    plan = lib.cwt_plan_create(2, 1000, 500.0, np.array([20.0]), np.array([10.0]), 0, lib.CWT_OUT_POWER, o)
+    try:
+        ep, n_in, n_o = lib.pack_epochs([1000, 600], 2, 1, 4)
+        x, p = torch.randn(n_in, device="cuda"), torch.zeros(n_o, device="cuda")
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        lib.cwt_execute_batch(plan, ep, x, None, p, None, s.cuda_stream)  # a prepared shape
+        torch.cuda.synchronize()
+        want = p.clone()
+        with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=s):
+            with pytest.raises(lib.CWTError):
+                lib.cwt_execute_batch(plan, ep, x, None, p, None, s.cuda_stream)
+        p.zero_()
+        lib.cwt_execute_batch(plan, ep, x, None, p, None)
+        assert torch.equal(p, want)
+    finally:
+        lib.cwt_plan_destroy(plan)
