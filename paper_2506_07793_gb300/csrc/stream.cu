@@ -45,6 +45,7 @@
 
 #include "fft_core.cuh"
 #include "internal.h"
+#include "zoom.cuh"
 
 namespace cwtk {
 namespace {
@@ -72,22 +73,36 @@ struct StreamItem {
 
 // One (hop, channel) per CTA: forward FFT of the window into shared memory,
 // then every scale's band product + inverse FFT, keeping the H centred outputs.
-__global__ void __launch_bounds__(kSThreads) stream_kernel(const StreamItem *__restrict__ items,
+//
+// Bound by instruction issue.  The inverse FFT, 2048 = 8 x 16 x 16, is done only
+// as far as its kept outputs need: pass 0 has one nonzero input per butterfly
+// where the band is no wider than a butterfly's stride (fft_pass0_sparse), and of
+// the last pass, which would give 2048 outputs, the H kept ones are formed as
+// sums of its 16 inputs.  800 channels at 250 ... 4000 Hz, H = 13 ... 200, 64
+// scales: 224 us, 316 with whole FFTs.
+__global__ void __launch_bounds__(kSThreads, 2) stream_kernel(const StreamItem *__restrict__ items,
                                                            const float2 *__restrict__ tw, int S) {
     constexpr int T = kSW / kSR;  // 128 threads per row
     constexpr int P = kSThreads / T;
+    using Shape = FftShape<kSW, kSR>;
+    constexpr int R0 = Shape::R0, G0 = Shape::G0, NS = R0;  // passes 0 (radix R0), 1 and 2 (radix 16)
+    static_assert(Shape::NP == 3 && R0 * kSR * kSR == kSW, "three passes");
     __shared__ float2 spec[kSW];
     extern __shared__ float2 ssm[];
     const StreamItem it = items[blockIdx.x];
     const int rl = threadIdx.x / T, j = threadIdx.x % T;
-    float2 *st = ssm + rl * FftShape<kSW, kSR>::SMEM_F2;
+    float2 *st = ssm + rl * Shape::SMEM_F2;
     // forward: only row-slot 0 holds data; the other slots transform zeros
     {
         const bool act = rl == 0;
+        const long long m = it.start % it.cap;
+        const int ring0 = (int)(m < 0 ? m + it.cap : m);  // the window's first sample in the ring; kSW <= cap
         auto load = [&](int i) -> float2 {
-            const long long a = it.start + i;
             float v = 0.f;
-            if (act && a >= 0) v = it.ring[a % it.cap];
+            if (act && it.start + i >= 0) {
+                const int q = ring0 + i;
+                v = it.ring[q >= it.cap ? q - it.cap : q];
+            }
             return make_float2(v, 0.f);
         };
         auto store = [&](int t, float2 v) {
@@ -97,6 +112,7 @@ __global__ void __launch_bounds__(kSThreads) stream_kernel(const StreamItem *__r
     }
     __syncthreads();
     const int lo = kSW - it.D - it.H;  // first kept window position
+    const int k1 = j & (NS - 1), base1 = (j - k1) * kSR + k1;
 #pragma unroll 1
     for (int s0 = 0; s0 < S; s0 += P) {
         const int s = s0 + rl;
@@ -111,12 +127,48 @@ __global__ void __launch_bounds__(kSThreads) stream_kernel(const StreamItem *__r
             }
             return make_float2(0.f, 0.f);
         };
+        float2 v[kSR];
+        if (B <= kSW / R0) {
+            auto first = [&](int jj, int &r, float2 &x) -> bool {
+                const int d0 = (jj - b0) & (kSW / R0 - 1);
+                if (d0 >= B) return false;
+                const int k = (b0 + d0) & (kSW - 1);
+                r = (k - jj) / (kSW / R0);
+                x = load(k);
+                return true;
+            };
+            fft_pass0_sparse<kSW, kSR, +1>(v, j, tw, first);
+        } else {
+            fft_pass0_dense<kSW, kSR, +1>(v, j, load);
+        }
+        __syncthreads();  // the previous row's outputs are formed
+#pragma unroll
+        for (int g = 0; g < G0; ++g)
+#pragma unroll
+            for (int r = 0; r < R0; ++r) *CWT_SMEM(&st[spad2((j + g * T) * R0 + r)]) = v[g * R0 + r];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSR; ++r) v[r] = *CWT_SMEM(&st[spad2(j + r * T)]);
+        twiddle_chain<kSR>(v, __ldg(&tw[k1 * (kTwN / (NS * kSR))]));
+        dft<kSR, +1>(v);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSR; ++r) *CWT_SMEM(&st[spad2(base1 + r * NS)]) = v[r];
+        __syncthreads();
         float *o = it.out + (size_t)(act ? s : 0) * it.H;
-        auto store = [&](int t, float2 v) {
-            const int q = t - lo;
-            if (act && q >= 0 && q < it.H) o[q] = fmaf(v.x, v.x, v.y * v.y);
-        };
-        fft_row<kSW, kSR, +1>(st, tw, j, load, store);
+#pragma unroll 1
+        for (int q = j; act && q < it.H; q += T) {
+            const int t = lo + q, jj = t & (T - 1);
+#pragma unroll
+            for (int r = 0; r < kSR; ++r) v[r] = *CWT_SMEM(&st[spad2(jj + r * T)]);
+            zoom_twiddle<kSR>(v, __ldg(&tw[t * (kTwN / kSW)]), __ldg(&tw[(8 * t & (kSW - 1)) * (kTwN / kSW)]));
+#pragma unroll
+            for (int h = kSR / 2; h >= 1; h /= 2)
+#pragma unroll
+                for (int r = 0; r < h; ++r) v[r] = make_float2(v[r].x + v[r + h].x, v[r].y + v[r + h].y);
+            const float re = v[0].x, im = v[0].y;
+            o[q] = fmaf(re, re, im * im);
+        }
     }
 }
 
