@@ -16,15 +16,16 @@
 //  * cwt_server_step gathers every ready hop of every open stream into one
 //    launch (continuous batching): streams that joined since the last step
 //    are simply in the next batch, and closed streams leave it.  Two batches
-//    may be in flight; results are copied to each stream's pinned host queue
-//    and a host callback stamps the completion time, so latency is measured
-//    from the moment a hop became ready to the moment its power is in host
-//    memory.
-//  * Admission: a stream is refused (CWT_EBUSY) when no slot is free or its
-//    device memory (ring + its share of the batch buffers) would exceed the
-//    server's budget.  The batch buffers of both in-flight slots are grown at
-//    admission to the bound of every open stream (kMaxPending hops each), so
-//    cwt_server_step never allocates.
+//    may be in flight; the kernel writes each stream's results to its pinned
+//    host queue over the host link (a step of 16 streams, 13 MB of results:
+//    1.48 ms with copies after the kernel, 1.39 without) and a host callback
+//    stamps the completion time, so latency is measured from the moment a hop
+//    became ready to the moment its power is in host memory.
+//  * Admission: a stream is refused (CWT_EBUSY) when no slot is free or what it
+//    counts (stream_dev_bytes) would exceed the server's budget.  The item
+//    tables of both in-flight slots are grown at admission to the bound of
+//    every open stream (kMaxPending hops each), so cwt_server_step never
+//    allocates.
 //  * Pushes copy into the rings on a copy stream of their own; each batch
 //    waits for an event recorded there, so a push never queues behind a batch
 //    in flight.  A push cannot overwrite ring samples that a batch in flight
@@ -63,7 +64,7 @@ double now_s() {
 
 struct StreamItem {
     const float *ring;  // channel row of the stream's ring
-    float *out;         // [S][H] block of this (hop, channel)
+    float *out;         // [S][H] block of this (hop, channel), in pinned host memory
     const float *bank;  // [S][W]
     const int *band;    // [S][2]
     long long start;    // absolute index of the window's first sample (may be < 0)
@@ -209,8 +210,6 @@ struct Bank {
 struct Slot {
     StreamItem *d_items = nullptr, *h_items = nullptr;
     size_t items_cap = 0;
-    float *d_out = nullptr;
-    size_t out_cap = 0;  // floats
     cudaEvent_t done = nullptr;
     bool busy = false;
     std::vector<std::pair<int, long long>> hops;  // (stream id, e) carried by this batch
@@ -238,7 +237,7 @@ struct cwt_server_s {
     cudaStream_t st = nullptr;   // the server's own CUDA stream (batches)
     cudaStream_t cst = nullptr;  // pushes into the rings
     cudaEvent_t pushed = nullptr;  // recorded on cst before each batch
-    size_t bound_items = 0, bound_out = 0;  // batch-buffer bound of the open streams
+    size_t bound_items = 0;  // items that the open streams can have in a batch
     std::string last_error;
 };
 
@@ -319,44 +318,33 @@ cudaError_t bank_for(cwt_server_s *srv, double fs, int *idx) {
     return cudaSuccess;
 }
 
-// Grow both slots' batch buffers to hold `items` work items and `outf`
-// output floats.  The new buffers are allocated first, so a failure leaves
-// every slot as it was; a slot's batch in flight is waited for before its
-// buffers are replaced.  Called at admission, never by cwt_server_step.
-cudaError_t grow_slots(cwt_server_s *srv, size_t items, size_t outf) {
+// Grow both slots' item tables to `items` work items.  The new tables are
+// allocated first, so a failure leaves every slot as it was; a slot's batch in
+// flight is waited for before its table is replaced.  Called at admission,
+// never by cwt_server_step.
+cudaError_t grow_slots(cwt_server_s *srv, size_t items) {
     for (Slot &sl : srv->slots) {
-        if (sl.items_cap >= items && sl.out_cap >= outf) continue;
+        if (sl.items_cap >= items) continue;
         StreamItem *d_items = nullptr, *h_items = nullptr;
-        float *d_out = nullptr;
-        cudaError_t e = cudaSuccess;
-        if (sl.items_cap < items) {
-            e = cwtk::dmalloc(&d_items, sizeof(StreamItem) * items);
-            if (e == cudaSuccess) e = cwtk::hmalloc(&h_items, sizeof(StreamItem) * items);
-        }
-        if (e == cudaSuccess && sl.out_cap < outf) e = cwtk::dmalloc(&d_out, sizeof(float) * outf);
+        cudaError_t e = cwtk::dmalloc(&d_items, sizeof(StreamItem) * items);
+        if (e == cudaSuccess) e = cwtk::hmalloc(&h_items, sizeof(StreamItem) * items);
         if (e == cudaSuccess && sl.busy) e = cudaEventSynchronize(sl.done);
         if (e != cudaSuccess) {
             cudaFree(d_items);
             if (h_items) cudaFreeHost(h_items);
-            cudaFree(d_out);
             return e;
         }
-        if (d_items) {
-            cudaFree(sl.d_items);
-            if (sl.h_items) cudaFreeHost(sl.h_items);
-            sl.d_items = d_items;
-            sl.h_items = h_items;
-            sl.items_cap = items;
-        }
-        if (d_out) {
-            cudaFree(sl.d_out);
-            sl.d_out = d_out;
-            sl.out_cap = outf;
-        }
+        cudaFree(sl.d_items);
+        if (sl.h_items) cudaFreeHost(sl.h_items);
+        sl.d_items = d_items;
+        sl.h_items = h_items;
+        sl.items_cap = items;
     }
     return cudaSuccess;
 }
 
+// What a stream counts against the server's budget: its ring and, in the
+// pinned queue that the kernel writes, the results of the batches in flight.
 size_t stream_dev_bytes(const cwt_server_s *srv, int C, int H) {
     const size_t ring = sizeof(float) * (size_t)C * (kSW + (size_t)kMaxPending * H);
     const size_t outs = sizeof(float) * (size_t)C * srv->S * H * kMaxPending * kSlots;
@@ -464,7 +452,6 @@ cwt_status cwt_server_destroy(cwt_server s) {
         }
         for (auto &sl : s->slots) {
             cudaFree(sl.d_items);
-            cudaFree(sl.d_out);
             if (sl.h_items) cudaFreeHost(sl.h_items);
             if (sl.done) cudaEventDestroy(sl.done);
         }
@@ -521,8 +508,7 @@ cwt_status cwt_stream_open(cwt_server s, int channels, double fs, int *stream_id
     if (e == cudaSuccess) e = cudaMemsetAsync(st.d_ring, 0, ring_b, s->cst);
     if (e == cudaSuccess) e = cwtk::hmalloc(&st.h_queue, q_b);
     const size_t items = s->bound_items + (size_t)channels * kMaxPending;
-    const size_t outf = s->bound_out + (size_t)channels * s->S * H * kMaxPending;
-    if (e == cudaSuccess) e = grow_slots(s, items, outf);
+    if (e == cudaSuccess) e = grow_slots(s, items);
     if (e != cudaSuccess) {
         cudaFree(st.d_ring);
         if (st.h_queue) cudaFreeHost(st.h_queue);
@@ -532,7 +518,6 @@ cwt_status cwt_stream_open(cwt_server s, int channels, double fs, int *stream_id
         return cuda_fail(s, e);
     }
     s->bound_items = items;
-    s->bound_out = outf;
     std::lock_guard<std::mutex> lk(s->mu);
     for (int i = st.queue_slots - 1; i >= 0; --i) st.free_slots.push_back(i);
     st.dev_bytes = need;
@@ -597,9 +582,6 @@ cwt_status cwt_server_step(cwt_server s, int *hops_launched) {
     }
     std::vector<StreamItem> items;
     std::vector<std::pair<int, long long>> hops;
-    std::vector<std::pair<size_t, size_t>> copies;  // (out offset floats, count) per hop
-    std::vector<float *> dsts;
-    size_t out_floats = 0;
     {
         std::lock_guard<std::mutex> lk(s->mu);
         if (sl.busy) return CWT_EAGAIN;
@@ -615,7 +597,7 @@ cwt_status cwt_server_step(cwt_server s, int *hops_launched) {
                 for (int c = 0; c < st.C; ++c) {
                     StreamItem it;
                     it.ring = st.d_ring + (size_t)c * st.cap;
-                    it.out = nullptr;  // filled once the buffer exists
+                    it.out = st.h_queue + (size_t)h.slot_out * blk + (size_t)c * s->S * st.H;
                     it.bank = s->banks[st.bank].bank;
                     it.band = s->banks[st.bank].band;
                     it.start = h.e - kSW;
@@ -623,11 +605,7 @@ cwt_status cwt_server_step(cwt_server s, int *hops_launched) {
                     it.H = st.H;
                     it.D = st.D;
                     items.push_back(it);
-                    (void)c;
                 }
-                copies.push_back({out_floats, blk});
-                dsts.push_back(st.h_queue + (size_t)h.slot_out * blk);
-                out_floats += blk;
                 hops.push_back({st.id, h.e});
                 st.inflight.push_back(h);
             }
@@ -635,25 +613,16 @@ cwt_status cwt_server_step(cwt_server s, int *hops_launched) {
     }
     if (hops_launched) *hops_launched = (int)hops.size();
     if (items.empty()) return CWT_OK;
-    // the slot buffers were sized at admission for kMaxPending hops of every
+    // the slot's table was sized at admission for kMaxPending hops of every
     // open stream, which bounds any batch: nothing is allocated here
-    if (items.size() > sl.items_cap || out_floats > sl.out_cap) {
-        s->last_error = "batch exceeds the buffers sized at admission";
+    if (items.size() > sl.items_cap) {
+        s->last_error = "batch exceeds the table sized at admission";
         return CWT_ECUDA;
     }
     // the batch reads samples pushed on the copy stream
     cudaError_t e = cudaEventRecord(s->pushed, s->cst);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s->st, s->pushed, 0);
     if (e != cudaSuccess) return cuda_fail(s, e);
-    // per-channel output blocks: hop block base + c * S * H
-    {
-        size_t i = 0;
-        for (size_t h = 0; h < copies.size(); ++h) {
-            const Stream &st = s->streams[hops[h].first];
-            for (int c = 0; c < st.C; ++c, ++i)
-                items[i].out = sl.d_out + copies[h].first + (size_t)c * s->S * st.H;
-        }
-    }
     std::memcpy(sl.h_items, items.data(), sizeof(StreamItem) * items.size());
     e = cudaMemcpyAsync(sl.d_items, sl.h_items, sizeof(StreamItem) * items.size(),
                         cudaMemcpyHostToDevice, s->st);
@@ -661,9 +630,6 @@ cwt_status cwt_server_step(cwt_server s, int *hops_launched) {
         stream_kernel<<<(unsigned)items.size(), kSThreads, kStreamSmem, s->st>>>(sl.d_items, s->tw, s->S);
         e = cudaGetLastError();
     }
-    for (size_t h = 0; h < copies.size() && e == cudaSuccess; ++h)
-        e = cudaMemcpyAsync(dsts[h], sl.d_out + copies[h].first, sizeof(float) * copies[h].second,
-                            cudaMemcpyDeviceToHost, s->st);
     if (e == cudaSuccess) {
         std::lock_guard<std::mutex> lk(s->mu);
         sl.hops = hops;
@@ -737,7 +703,6 @@ cwt_status cwt_stream_close(cwt_server s, int id) {
         queue = st.h_queue;
         s->dev_bytes -= st.dev_bytes;
         s->bound_items -= (size_t)st.C * kMaxPending;
-        s->bound_out -= (size_t)st.C * s->S * st.H * kMaxPending;
         st = Stream();
     }
     cudaFree(ring);
