@@ -108,6 +108,8 @@ struct cwt_plan_s {
     // host-buffer execution staging (allocated on first use)
     void *stage_in = nullptr, *stage_c = nullptr, *stage_p = nullptr, *stage_ph = nullptr;
     size_t stage_bytes = 0;
+    cudaStream_t copy_stream = nullptr;  // copies of a host transform's slices, with sliced
+    cudaEvent_t sliced = nullptr;
 
     cwtk::BatchState *batch = nullptr;  // batch path state (banks per length, graph, tuning)
 
