@@ -394,7 +394,7 @@ def run_batch(args):
     alg_bytes = int(x_host.nbytes) + coeffs * 4 + int(stats.bank_bytes)
     k_s = ms_b / max(n_b, 1) * 1e-3
     achieved = alg_bytes / k_s / 1e9
-    roofline = {"kernel": "batch_kernel (persistent, CUDA graph)", "bound": "hbm",
+    roofline = {"kernel": "batch kernels (forward FFTs, residue classes; all launches of a batch)", "bound": "hbm",
                 "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "peak_source": peak_kind, "traffic": None,
                 "alg_bytes_per_launch": alg_bytes, "kernel_ms": k_s * 1e3}
@@ -429,8 +429,7 @@ def run_batch(args):
                        "decimation": d, "coefficients_per_step": coeffs,
                        "l2": "inputs (2.2 GB) and outputs (35 GB) exceed L2; 256 MB buffer also "
                              "overwritten between timed steps",
-                       "autotuned": {"inverse_radix": stats.inverse_radix, "order": stats.order,
-                                     "candidate_ms": list(stats.tune_ms)},
+                       "schedule": {"inverse_radix": stats.inverse_radix, "order": stats.order},
                        "items": stats.items, "grid": stats.grid, "wall_s_timed_region": wall,
                        "parallelism": f"weak x{world}, no collective"},
             "roofline": roofline, "e2e": e2e, "gpu_launches": args.steps, "clocks": clk,
@@ -1100,7 +1099,8 @@ def run_plan_workload(args, name):
                  "FP32 accumulation)")
     else:
         kname = f"cl_scale_block_kernel<{N},float> (cluster of {N // 16384} CTAs)"
-    roofline = {"kernel": kname, "bound": "hbm",
+    # narrow bands run by residue classes, the rest (if any) on the kernel named above
+    roofline = {"kernel": "scale blocks: zoom_kernel / zoom_row_kernel / wide_*_kernel, " + kname, "bound": "hbm",
                 "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "peak_source": peak_kind,
                 "traffic": traffic if name == "fused" else None,
@@ -1203,8 +1203,8 @@ def finish_plan_line(args, name, w, info, N, world, rank, value, ms_step, wall, 
             "roofline": roofline,
             "e2e": e2e,
             "plain_fp32_gpu": plain,
-            # forward FFT + scale block per step (+ the spectrum bounds of the tensor-core path)
-            "gpu_launches": (3 if args.precision != "fp32" else 2) * args.steps,
+            # at least: forward FFT + scale block per step; residue classes take further launches
+            "gpu_launches": 2 * args.steps,
             "clocks": clk,
         }
         if e2e is None:

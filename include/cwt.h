@@ -122,7 +122,7 @@ typedef enum {
     CWT_KERNEL_BANK = 0,        /* wavelet-bank + band generation (plan creation) */
     CWT_KERNEL_FORWARD_FFT = 1, /* per-channel forward FFT */
     CWT_KERNEL_SCALE_BLOCK = 2, /* fused multiply + inverse FFT + reduce + store */
-    CWT_KERNEL_BATCH = 3,       /* persistent batch kernel (one graph launch) */
+    CWT_KERNEL_BATCH = 3,       /* a batch's kernels */
     CWT_KERNEL_COUNT = 4
 } cwt_kernel_id;
 
@@ -141,15 +141,16 @@ typedef struct {
 /* What the batch path did last (cwt_plan_batch_stats). */
 typedef struct {
     int items;              /* work items (epoch, channel group) of the last batch */
-    int grid;               /* persistent CTAs launched */
-    int inverse_radix;      /* autotuned points per thread of the inverse FFTs (16 or 32) */
-    int order;              /* autotuned item order: 0 largest FFT first, 1 input order */
-    int tuned;              /* 1 once the autotuner has chosen for this batch shape */
+    int grid;               /* CTAs of the persistent kernel */
+    int inverse_radix;      /* points per thread of its inverse FFTs: 16, or 32 where a row needs it */
+    int order;              /* item order: 0, largest FFT first */
+    int tuned;              /* 1 once the batch shape is prepared */
     int reserved;
-    double tune_ms[4];      /* candidate times: (16,0), (32,0), (16,1), (32,1); -1 for a
-                               radix-16 candidate the batch rules out (an inverse row
-                               longer than 4096 points, at N_e = 8192 and odd d) */
-    long long graph_launches;
+    double tune_ms[4];      /* schedules (16,0), (32,0), (16,1), (32,1): 0, or -1 for a
+                               radix-16 one that the batch rules out (an inverse row
+                               longer than 4096 points, at N_e = 8192 and odd d);
+                               the schedule is a rule, nothing is timed */
+    long long graph_launches; /* forward launches, one per workspace of a batch */
     size_t bank_bytes;      /* device bytes of the per-length wavelet banks */
 } cwt_batch_stats;
 
@@ -160,7 +161,8 @@ typedef struct {
                        accumulation (the Cooley-Tukey factorisation of Section
                        "Fast Fourier transform"; error within 2e-3 of the row's
                        peak power): power-of-two N of 16384 ... 131072 only (else
-                       CWT_EUNSUPPORTED); not for cwt_execute_batch */
+                       CWT_EUNSUPPORTED); not for cwt_execute_batch.  Scales whose
+                       band is narrow run in FP32, which is faster there */
     int decimation; /* keep every d-th output sample, d >= 1 (default 1) */
     int pad_policy; /* cwt_pad_policy (default CWT_PAD_POW2) */
     int fft_length; /* 0: from pad_policy; else an explicit N >= samples that is a
@@ -362,8 +364,10 @@ cwt_status cwt_execute(cwt_plan plan, const void *d_signal, void *d_complex, voi
  * for the outputs.  An output buffer in page-locked host memory that the
  * device can address (cudaHostAlloc / cudaMallocHost, cudaHostRegister with
  * mapping, e.g. torch pin_memory(); 16-byte aligned) is written directly by
- * the kernels' epilogues over the host link, with no staging copy; any other
- * output goes to a device staging buffer and is copied back.  Staging buffers
+ * the kernels' epilogues over the host link, with no staging copy, unless the
+ * outputs exceed 48 MB and the plan runs scales by residue classes: those are
+ * staged and copied in slices of channels while the next are computed.  Any
+ * other output goes to a device staging buffer and is copied back.  Staging buffers
  * are allocated on the first call and kept by the plan.  Same layouts as
  * cwt_execute.  Returns when the outputs are in host memory.
  */
@@ -371,20 +375,21 @@ cwt_status cwt_execute_host(cwt_plan plan, const void *h_signal, void *h_complex
                             void *h_phase, void *stream);
 
 /*
- * cwt_execute_batch -- many epochs of uneven length in one persistent launch
- * replayed from a CUDA graph.  Epoch e is the same transform as cwt_execute
+ * cwt_execute_batch -- many epochs of uneven length in one call, a few
+ * launches for all of them.  Epoch e is the same transform as cwt_execute
  * on its own samples (padded length N_e = next power of two >= max(n_e, 32),
  * or >= n_e + R + 1 with CWT_EDGE_LINEAR,
  * Section "Fast Fourier transform"), with the plan's channels, scales,
  * decimation and output kinds.  The paper loops over recordings in Python
- * (Section "Wavelength and flexibility"); here they share one launch.
+ * (Section "Wavelength and flexibility"); here they share the launches.
  *   epochs[n_epochs]  host array of cwt_epoch (offsets in elements)
  *   d_in              device packed float32 input
  *   d_complex / d_power / d_phase  device packed outputs (exactly the plan's kinds)
  * Requires an F32 plan.  The first batch of a new shape generates the banks
- * for its lengths (allocating and waiting) and runs the autotuner, which times
- * four schedules on this batch and keeps the fastest; later batches of the
- * same shape only replay the graph.  Asynchronous on `stream` otherwise.
+ * for its lengths and a workspace for the spectra's kept bins, up to 256 MB or
+ * one epoch's (allocating and waiting); later batches of the same shape only
+ * launch.  Asynchronous on `stream` otherwise.  Not inside a stream capture
+ * (CWT_ECUDA).
  * CWT_EUNSUPPORTED for F64 plans, smooth-padded plans, or epochs whose
  * padded length would exceed 8192 samples.  CWT_EINVAL (before any device
  * work) when an epoch's N_e cannot represent one of the plan's scales (the
@@ -556,13 +561,12 @@ cwt_status cwt_measure_peak(int what, double *tflops);
  * before any device work.
  * The first call on a device (the current device) resolves the array's device
  * address and writes its twiddle table, then waits for that on `stream`.  No
- * call may be made inside a stream capture: each one copies freqs_hz and
- * n_cycles from pageable host memory (cudaMemcpyAsync), which a captured
- * stream refuses or would replay from host memory the caller may have freed.
+ * call may be made inside a stream capture (CWT_ECUDA): a graph would replay
+ * into the shared array at times that its caller does not order.
  * The address is kept for the
  * life of the process: do not call this entry point again on a device after
- * cudaDeviceReset.  Every call copies freqs_hz and n_cycles into the array
- * (so the caller may reuse them as soon as the call returns), reuses the same
+ * cudaDeviceReset.  Every call passes up to 128 scales on by value and
+ * copies more from the host (so the caller may reuse them as soon as the call returns), reuses the same
  * array and overwrites everything it reads, so nothing needs clearing between
  * calls; calls that overlap on the GPU (unordered streams, other host
  * threads) race on it and must be serialised by the caller.  Its kernels run
