@@ -209,7 +209,7 @@ double whole_cost(int i, const ZoomShape &z) {
 // Cost of one row (ps) with first radix i and remaining length j of
 // zoom_wide.cuh (mean of power only and complex and power, launch by launch
 // over 38 rows of 131072 points less the launches' ends: first kernel 1.4 ps
-// per point, second 8 x 32 2.1, 16 x 32 2.4).
+// per point, second 16 x 16 2.1, 16 x 32 2.4).
 double wide_cost(int i, int j, const ZoomShape &z) {
     const WideInst &w = wide_rest(j);
     const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i);

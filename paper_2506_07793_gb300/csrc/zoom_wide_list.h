@@ -8,7 +8,6 @@
 #define CWT_WIDE_FIRST(X) \
     X(0, 2) X(1, 3) X(2, 4) X(3, 5) X(4, 6) X(5, 7) X(6, 8) X(7, 9) X(8, 10) X(9, 12) X(10, 14) X(11, 15) X(12, 16) X(13, 18) X(14, 20) X(15, 21) X(16, 24) X(17, 25) X(18, 27) X(19, 28) X(20, 30) X(21, 32)
 #define CWT_WIDE_REST_0(X) \
-    X(41, 8, 32, 16, 128, 5) \
     X(0, 16, 16, 16, 128, 5) \
     X(4, 16, 20, 16, 128, 4) \
     X(8, 15, 24, 16, 128, 4) \
@@ -19,7 +18,7 @@
     X(28, 20, 28, 16, 128, 2) \
     X(32, 25, 25, 16, 256, 2) \
     X(36, 25, 27, 16, 256, 2) \
-    X(40, 32, 32, 8, 256, 2)
+    X(14, 32, 32, 8, 256, 2)
 #define CWT_WIDE_REST_1(X) \
     X(1, 15, 18, 16, 128, 4) \
     X(5, 18, 18, 16, 128, 4) \
@@ -35,7 +34,6 @@
     X(2, 12, 24, 16, 128, 4) \
     X(6, 14, 24, 16, 128, 4) \
     X(10, 14, 27, 16, 128, 4) \
-    X(14, 20, 20, 16, 128, 3) \
     X(18, 21, 21, 16, 128, 3) \
     X(22, 18, 27, 16, 128, 3) \
     X(26, 21, 25, 16, 128, 2) \
@@ -56,5 +54,5 @@
 #define CWT_WIDE_REST(X) CWT_WIDE_REST_0(X) CWT_WIDE_REST_1(X) CWT_WIDE_REST_2(X) CWT_WIDE_REST_3(X)
 
 namespace cwtk {
-constexpr int kWideFirst = 22, kWideRest = 42;
+constexpr int kWideFirst = 22, kWideRest = 40;
 }
