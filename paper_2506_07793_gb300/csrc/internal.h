@@ -111,7 +111,7 @@ struct cwt_plan_s {
     cudaStream_t copy_stream = nullptr;  // copies of a host transform's slices, with sliced
     cudaEvent_t sliced = nullptr;
 
-    cwtk::BatchState *batch = nullptr;  // batch path state (banks per length, graph, tuning)
+    cwtk::BatchState *batch = nullptr;  // batch path state (banks per length, workspace, graph)
 
     bool profiling = false;
     std::vector<cwtk::ProfEvent> prof, prof_pool;
