@@ -5,8 +5,8 @@ headers of the plan-time compiler embedded as a generated jit_headers.cpp, then
 linked into paper_2506_07793_gb300/_lib/libcwt_gb300.so (static CUDA runtime;
 NVRTC from the toolkit, found through an rpath; the driver's module calls are
 fetched at run time through the runtime).  Objects go
-to paper_2506_07793_gb300/_build/.  A source is rebuilt when it, or any header
-under csrc/ or include/, is newer than its object.
+to paper_2506_07793_gb300/_build/.  A source is rebuilt when it, any header
+under csrc/ or include/, or this file (the flags) is newer than its object.
 """
 import concurrent.futures as cf
 import glob
@@ -39,7 +39,7 @@ def nvcc():
 
 def _headers():
     return glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
-        glob.glob(os.path.join(ROOT, "include", "*.h"))
+        glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
 
 
 def _compile(src, extra, verbose, bdir=BUILD, defs=()):
@@ -115,7 +115,10 @@ def build(force=False, verbose=False, extra_flags=(), check=False):
         for o in glob.glob(os.path.join(bdir, "*.o")):
             os.remove(o)
     extra = list(extra_flags) + (["-Xptxas", "-v"] if verbose else [])
-    defs = ["-DCWT_BOUNDS_CHECK"] if check else []
+    # The checked variant's device code is compressed (library 232 -> 32 MB): with
+    # both builds and their objects the tree passed 700 MB, too much to ship.  The
+    # ordinary one is not: unpacking would add 17 ms to a process's first call.
+    defs = ["-DCWT_BOUNDS_CHECK", "--compress-mode=size"] if check else []
     with cf.ThreadPoolExecutor(max_workers=min(len(srcs), os.cpu_count() or 4)) as ex:
         results = list(ex.map(lambda s: _compile(s, extra, verbose, bdir, defs), srcs))
     objs = [o for o, _ in results]
