@@ -196,7 +196,13 @@ typedef struct {
                           environment variable CWT_JIT_CACHE_DIR naming a
                           writable directory, also on disk, and later processes
                           load them instead of compiling */
-    int reserved[6];
+    int whole_rows;    /* 1: every scale is transformed as a whole row, on the kernels
+                          that `precision` and `specialize` name.  0 (default):
+                          float32 plans run a scale by the residue classes of its
+                          output samples, in FP32, where that is faster -- narrow
+                          bands at any length, wide ones at most lengths
+                          (cwt_plan_routes says how many).  Other values read as 0 */
+    int reserved[5];
 } cwt_options;
 
 typedef struct {
@@ -336,6 +342,14 @@ cwt_status cwt_plan_destroy(cwt_plan plan);
 
 /* Describe the plan (host-only, no synchronisation). */
 cwt_status cwt_plan_info(cwt_plan plan, cwt_plan_info_t *info);
+
+/* How cwt_execute transforms the plan's scales (host-only, no synchronisation):
+ * *whole_rows of them as whole rows, on the kernels that cwt_plan_info describes
+ * (its precision, radices, fixed_kernel, cluster and specialized fields),
+ * *classes by output residue classes in one kernel and *two_kernels in two, both
+ * in FP32.  The three add up to the plan's scales.  Outputs are host memory owned
+ * by the caller.  CWT_EINVAL for a NULL argument. */
+cwt_status cwt_plan_routes(cwt_plan plan, int *whole_rows, int *classes, int *two_kernels);
 
 /* Device bytes owned by the plan (0 for NULL). */
 size_t cwt_plan_workspace_bytes(cwt_plan plan);

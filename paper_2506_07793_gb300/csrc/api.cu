@@ -332,6 +332,7 @@ cwt_status cwt_plan_create(cwt_plan *out, int channels, int samples, double fs,
     p->pad_extra = pad_extra;
     p->norm2 = o.normalization == CWT_NORM_MNE ? 2.0 : 1.0;
     p->outputs = output_kinds;
+    p->whole_rows = o.whole_rows == 1;
     p->io = o.io_dtype;
     p->freqs.assign(freqs_hz, freqs_hz + n_freqs);
     p->cycles.assign(n_cycles, n_cycles + n_freqs);
@@ -470,6 +471,13 @@ cwt_status cwt_plan_info(cwt_plan p, cwt_plan_info_t *info) {
         info->fixed_kernel = 1;
         info->inlined_pair[0] = info->inlined_pair[1] = 0;
     }
+    return CWT_OK;
+}
+
+cwt_status cwt_plan_routes(cwt_plan p, int *whole_rows, int *classes, int *two_kernels) {
+    if (!p || !whole_rows || !classes || !two_kernels) return CWT_EINVAL;
+    *whole_rows = p->rest_scales;
+    cwtk::zoom_routes(p->zoom, classes, two_kernels);
     return CWT_OK;
 }
 

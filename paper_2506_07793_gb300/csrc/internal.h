@@ -54,6 +54,7 @@ inline const float2 *twiddles_pow2(const float2 *tw, int L) { return tw + 2 * kT
 
 struct ZoomPlan;  // zoom.cu
 void free_zoom_plan(ZoomPlan *z);
+void zoom_routes(const ZoomPlan *z, int *classes, int *two_kernels);  // scales of each form
 
 struct BatchState;
 void free_batch_state(BatchState *b);
@@ -101,6 +102,7 @@ struct cwt_plan_s {
     const float2 *tw = nullptr;
     cwtk::ZoomPlan *zoom = nullptr;   // scales run by output residue classes (zoom.cu), or null
     int rest_scales = 0;              // the other scales: how many, and which (null: all S)
+    bool whole_rows = false;          // cwt_options.whole_rows
     int *rest_list = nullptr;
     size_t bytes = 0;
     double bank_ms = 0;

@@ -472,6 +472,12 @@ void free_zoom_plan(ZoomPlan *z) {
     delete z;
 }
 
+void zoom_routes(const ZoomPlan *z, int *classes, int *two_kernels) {
+    *classes = *two_kernels = 0;
+    if (z)
+        for (const ZoomClass &c : z->classes) (c.wide >= 0 ? *two_kernels : *classes) += c.ns;
+}
+
 static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     const int S = p->S;
     const int f = std::gcd(p->N, p->d), M = p->N / f;
@@ -540,7 +546,7 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
 cudaError_t zoom_plan_create(cwt_plan_s *p, cudaStream_t st) {
     p->rest_scales = p->S;
     // double outputs keep the whole-row kernels' bits
-    if (p->io != CWT_DTYPE_F32) return cudaSuccess;
+    if (p->io != CWT_DTYPE_F32 || p->whole_rows) return cudaSuccess;
     try {
         return zoom_plan_build(p, st);
     } catch (const std::bad_alloc &) {

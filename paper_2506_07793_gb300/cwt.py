@@ -40,7 +40,8 @@ class cwt_options(ctypes.Structure):
                 ("pad_policy", ctypes.c_int), ("fft_length", ctypes.c_int),
                 ("io_dtype", ctypes.c_int), ("edge_mode", ctypes.c_int),
                 ("gmw_gamma", ctypes.c_double), ("normalization", ctypes.c_int),
-                ("specialize", ctypes.c_int), ("reserved", ctypes.c_int * 6)]
+                ("specialize", ctypes.c_int), ("whole_rows", ctypes.c_int),
+                ("reserved", ctypes.c_int * 5)]
 
 
 class cwt_plan_info_t(ctypes.Structure):
@@ -109,6 +110,7 @@ _sig("cwt_plan_create", ctypes.c_int,
       ctypes.c_int, ctypes.c_uint, ctypes.POINTER(cwt_options)])
 _sig("cwt_plan_destroy", ctypes.c_int, [_vp])
 _sig("cwt_plan_info", ctypes.c_int, [_vp, ctypes.POINTER(cwt_plan_info_t)])
+_sig("cwt_plan_routes", ctypes.c_int, [_vp, _ip, _ip, _ip])
 _sig("cwt_plan_workspace_bytes", ctypes.c_size_t, [_vp])
 _sig("cwt_plan_last_error", ctypes.c_char_p, [_vp])
 _sig("cwt_execute", ctypes.c_int, [_vp, _vp, _vp, _vp, _vp, _vp])
@@ -252,6 +254,13 @@ def cwt_plan_info(plan):
     return info
 
 
+def cwt_plan_routes(plan):
+    """(whole rows, by residue classes in one kernel, in two): scales of each form."""
+    n = [ctypes.c_int(0) for _ in range(3)]
+    _check(_lib.cwt_plan_routes(plan, *(ctypes.byref(i) for i in n)), "cwt_plan_routes")
+    return tuple(i.value for i in n)
+
+
 def cwt_plan_workspace_bytes(plan):
     return int(_lib.cwt_plan_workspace_bytes(plan))
 
@@ -364,8 +373,9 @@ class CWT:
     def __init__(self, channels, samples, fs, freqs, n_cycles, outputs=("power",),
                  wavelet="morlet", dtype="f32", decimation=1, fft_length=0, pad="pow2",
                  gmw_gamma=3.0, edge="cyclic", precision="fp32", normalization="unit",
-                 specialize=False):
+                 specialize=False, whole_rows=False):
         opt = cwt_options_init()
+        opt.whole_rows = int(bool(whole_rows))
         opt.normalization = {"unit": CWT_NORM_UNIT_ENERGY, "mne": CWT_NORM_MNE}[normalization]
         opt.specialize = int(specialize)  # False / True / 2 (tune)
         opt.precision = {"fp32": CWT_PREC_FP32, "tc_fp16": CWT_PREC_TC_FP16,
