@@ -385,6 +385,7 @@ cwt_status cwt_plan_create(cwt_plan *out, int channels, int samples, double fs,
             p->bytes += sizeof(float2) * (size_t)NL;
         }
     }
+    p->compiled = p->jit || tune;
     if (e == cudaSuccess) e = cwtk::launch_bank(p, st);
     if (e == cudaSuccess) e = cwtk::zoom_plan_create(p, st);
     if (e == cudaSuccess && tc) {

@@ -191,7 +191,6 @@ cudaError_t make_length(cwt_plan_s *p, int L, cudaStream_t st, BatchLength *out)
     if (e == cudaSuccess) {
         const int f = std::gcd(N, p->d);
         ZoomShape sh;
-        sh.N = N;
         sh.M = l.M = N / f;
         sh.sub = p->d / f;
         sh.n_out = 0;  // epochs of any length
@@ -205,7 +204,8 @@ cudaError_t make_length(cwt_plan_s *p, int L, cudaStream_t st, BatchLength *out)
         sh.rows_only = true;
         sh.wide = false;
         sh.channels = 4096;  // epochs x channels
-        sh.row_bytes = 0;
+        sh.both = false;
+        sh.compiled_cost = 0;
         zoom_select(sh, S, band.data(), &l.classes, &list, &rest);
         l.nrest = (int)rest.size();
         if (!list.empty()) {

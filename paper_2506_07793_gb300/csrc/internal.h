@@ -103,6 +103,7 @@ struct cwt_plan_s {
     cwtk::ZoomPlan *zoom = nullptr;   // scales run by output residue classes (zoom.cu), or null
     int rest_scales = 0;              // the other scales: how many, and which (null: all S)
     bool whole_rows = false;          // cwt_options.whole_rows
+    bool compiled = false;            // whole rows run on kernels compiled at the plan's creation
     int *rest_list = nullptr;
     size_t bytes = 0;
     double bank_ms = 0;

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -177,19 +178,25 @@ cudaError_t ensure_wide_smem(int i, int mode) {
 
 // Cost of one row (ps) on instance i by columns.  A run of R outputs starts at
 // a multiple of R past the row's base: unless 8 divides both, its ends share
-// 32-byte sectors with runs stored by other instructions, and sectors written
-// in part cost L2 a read once the outputs of a launch exceed it (complex and
-// power of 32 Mi points, 8 x 16: 2.02 ps per point at R = 64, 2.09 at 40, 3.29
-// at 50, 3.68 at 63; 16 x 16: 2.16, 2.29, 4.03, 4.52).  Column groups that
-// meet several rows form more band products.
-double column_cost(int i, const ZoomShape &z, int S) {
+// 32-byte sectors with runs stored by other instructions.  With one output array
+// that costs next to nothing (480 MB of power or of complex values: 0.95 of the
+// instance's cost aligned, 1.0 not); with two, whose sectors compete for L2, it
+// costs 1.25 at multiples of 4 and 1.3 ... 1.8 off them, against 1.15 (medians of
+// 2200 launches of 40 Mi points at 39 lengths, by columns per CTA and residues).
+double column_cost(int i, const ZoomShape &z) {
     const int R = z.M / inst(i).Q, P = inst(i).P;
-    const bool large = z.channels * S * z.row_bytes > 192e6;
-    double f = 1.0;
-    if (P > 4 && (R % 8 != 0 || z.n_out % 8 != 0)) f = large ? (R % 4 == 0 && z.n_out % 4 == 0 ? 1.3 : 1.7) : 1.15;
-    if (P > 4 && R < 8) f = R % 4 == 0 ? 1.35 : 1.9;
-    if (R % P != 0 && P % R != 0) f *= 1.1;
-    if (z.sub != 1) f *= 1.4;  // a division per output
+    const bool eighth = R % 8 == 0 && z.n_out % 8 == 0, quarter = R % 4 == 0 && z.n_out % 4 == 0;
+    const bool three = inst(i).Q / inst(i).QA != inst(i).LAST;  // passes
+    double f;
+    if (P <= 4) f = !z.both ? 0.92 : quarter ? 1.05 : 1.35;
+    else if (!z.both) f = eighth ? 0.95 : R >= 32 ? 1.0 : 1.1;
+    else if (quarter) f = eighth ? 1.15 : 1.25;
+    else if (P <= 8) f = three ? 1.35 : R >= 8 ? 1.95 : 1.35;
+    else f = P <= 16 ? 1.85 : R >= 128 ? 1.3 : R >= 64 ? 1.45 : 1.75;
+    if (R % P != 0 && P % R != 0) f *= 1.05;  // column groups that meet several rows form more band products
+    // a division per output, and fewer of them stored
+    if (z.sub != 1) f = three ? 1.25 : z.both ? 1.75 : 1.45;
+    if ((P > 8 || (P > 4 && z.sub != 1)) && R < 8) f *= 1.4;
     return (double)z.M * inst(i).cost * f;
 }
 
@@ -197,29 +204,34 @@ double column_cost(int i, const ZoomShape &z, int S) {
 // more where every row's band product serves few residues (8 x 16, power:
 // 1.74 ps per point at R = 32, 1.84 at 16, 1.88 at 8, 2.06 at 4, 2.57 at 2)
 // and where rows start off a sector, the more the fewer the slots of the last
-// pass (1.93, 2.07, 2.21, 2.57, 3.36).
+// pass (1.93, 2.07, 2.21, 2.57, 3.36); 1.2 of that with two output arrays.
 double whole_cost(int i, const ZoomShape &z) {
     const int R = z.M / inst(i).Q, J = z.M / inst(i).LAST;
     double f = 1.12 + 1.0 / R;
     if (z.n_out % 8 != 0 || z.n_out == 0) f += 0.08 + 6.0 / J;
     if (z.sub != 1) f *= 1.4;
+    else if (z.both) f *= 1.2;
     return (double)z.M * inst(i).cost * f;
 }
 
 // Cost of one row (ps) with first radix i and remaining length j of
-// zoom_wide.cuh (mean of power only and complex and power, launch by launch
-// over 38 rows of 131072 points less the launches' ends: first kernel 1.4 ps
-// per point, second 16 x 16 2.1, 16 x 32 2.4).
+// zoom_wide.cuh, as above: 2500 launches of 40 ... 120 Mi points at 39 lengths
+// within 7% rms for one output array, 10% for two.  The first kernel's stores are
+// runs of R = M / Q points: 1.8 ps per point at R >= 16, 2.3 at 8, 3.1 at 4, 5.6
+// at 2, 10.4 at 1 (QA = 16), where the whole-row kernels are the better ones.
 double wide_cost(int i, int j, const ZoomShape &z) {
     const WideInst &w = wide_rest(j);
-    const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i);
-    double f = Rp % 8 == 0 && z.n_out % 8 == 0 ? 1.0 : Rp % 4 == 0 && z.n_out % 4 == 0 ? 1.2 : 1.5;
-    if (z.sub != 1) f *= 1.4;
+    const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i), R = Rp / QA;
+    const bool eighth = Rp % 8 == 0 && z.n_out % 8 == 0, quarter = Rp % 4 == 0 && z.n_out % 4 == 0;
+    double f = z.both ? (eighth ? 1.15 : quarter ? 1.25 : 1.75) : eighth ? 0.95 : 1.0;
+    if (z.sub != 1) f = 1.6;
     const double pad = (double)((Rp + w.P - 1) / w.P * w.P) / Rp;
-    const double first = QA <= 8 ? 1.4 : 1.4 + 0.025 * (QA - 8) + (QA > 16 ? 0.02 * (QA - 16) : 0.0);
+    const double first = (QA <= 8 ? 1.4 : 1.4 + 0.025 * (QA - 8) + (QA > 16 ? 0.02 * (QA - 16) : 0.0)) +
+                         0.58 * std::min(QA, 16) * std::pow((double)R, -1.15);
     const double rest = 1.95 + 0.0007 * (w.QB * w.QC) + ((w.QB % 5 == 0 || w.QB % 7 == 0 || w.QB % 3 == 0) ? 0.15 : 0.0) +
                   ((w.QC % 5 == 0 || w.QC % 7 == 0 || w.QC % 3 == 0) ? 0.15 : 0.0)  + (w.P < 16 ? 0.1 : 0.0);
-    return (double)z.M * (first + rest * f * pad);
+    // and the wait of the second kernel for the first, shared by about ten scales
+    return (double)z.M * (first + rest * f * pad) + 4e5 / z.channels;
 }
 
 constexpr int kWideCode = 1 << 20;  // candidate codes of zoom_select: + 1024 i + j
@@ -251,7 +263,7 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
         const int R = z.M / inst(i).Q, cap = inst(i).Q - (inst(i).NB - 1);  // the window starts at a multiple of NB
         // few residues leave a row's band product little use and its stores short
         if (!z.rows_only && (R >= 4 || inst(i).P <= 4) && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem)
-            all.push_back({2 * i, column_cost(i, z, S), cap});
+            all.push_back({2 * i, column_cost(i, z), cap});
         if (!z.phase && R >= 2 && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
             row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(i, rows_per_cta(i, z.M, R), R), R) <= kMaxSmem)
             all.push_back({2 * i + 1, whole_cost(i, z), cap});
@@ -269,7 +281,7 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
     for (const Cand &c : all)
         if (open.empty() || c.cap > open.back().cap) open.push_back(c);
     // every scale on its cheapest transform, then classes dissolved into the
-    // remaining ones while the launch they save (3 us) outweighs the dearer
+    // remaining ones while the launches they save (3 us, 10 for two kernels) outweigh the dearer
     // transforms of their scales, at a nominal number of channels
     auto assign = [&](const std::vector<Cand> &o, std::vector<int> *to) -> double {
         double total = 0;
@@ -282,7 +294,8 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
             used[k] = 1;
             if (to) (*to)[(size_t)s] = o[k].code;
         }
-        for (char u : used) total += u ? 3e6 : 0.0;
+        for (size_t k = 0; k < o.size(); ++k)
+            if (used[k]) total += o[k].code >= kWideCode ? 10e6 : 3e6;  // two kernels, the second after the first
         return total;
     };
     std::vector<int> to((size_t)S, kRest);
@@ -305,6 +318,20 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
         if (drop == open.size()) break;
         open.erase(open.begin() + (long)drop);
         total = assign(open, &to);
+    }
+    // rows compiled for the plan: scales whose class is dearer join them, if that
+    // outweighs a launch of theirs alone
+    if (z.compiled_cost > 0) {
+        const bool rows = std::find(to.begin(), to.end(), kRest) != to.end();
+        double gain = rows ? 3e6 : 0.0;
+        std::vector<int> moved = to;
+        for (const Cand &c : open)
+            for (int s = 0; s < S; ++s)
+                if (to[(size_t)s] == c.code && c.code != kRest && c.cost > z.compiled_cost) {
+                    gain += z.channels * (c.cost - z.compiled_cost);
+                    moved[(size_t)s] = kRest;
+                }
+        if (gain > 3e6) to = moved;
     }
     for (const Cand &cand : open) {
         const int k = cand.code;
@@ -439,16 +466,26 @@ namespace {
 // MB, 1.69 with 40, 1.61 with 57, 1.67 with 80, 1.62 with 400).
 constexpr size_t kWideBytes = (size_t)56 << 20;
 
-// Cost of one row (ps) on the whole-row kernels that are compiled in (a plan
-// with kernels compiled at its creation takes the same split of its scales).
-double row_cost(const cwt_plan_s *p) {
-    if (p->precision != CWT_PREC_FP32) return (double)p->N * 10.0;  // tensor-core stages: 340 us per 1024 x 32768
-    // the rest are wide bands, whose first pass is dense: 64 x 10000, 20 of 100
-    // scales, complex and power: 5.6 ps per point at 16384, 4.4 at 10000
-    if (!p->mr) return (double)p->M * (p->M <= kMaxFft ? 4.4 : 7.4);
-    if (p->cl > 1) return (double)p->N * (p->sch.fixed_cl >= 0 ? 7.2 : 30.0);
-    // (entered below that: on odd radices the two-kernel form takes 6.3 where its model says 4.1)
-    return (double)p->N * (p->sch.fixed >= 0 ? 3.7 : p->sch.fast >= 0 ? 6.5 : 14.0);
+// Cost of one row (ps) on the whole-row kernels, for the bands that are left to
+// them: wide ones, whose first pass is dense (medians of power alone and of
+// complex and power, 40 Mi points; a narrow band takes 0.75 ... 0.9 of it); or on
+// kernels compiled at the plan's creation, for lengths without compiled-in ones.
+double row_cost(const cwt_plan_s *p, bool both, bool compiled) {
+    if (p->precision != CWT_PREC_FP32)  // tensor-core stages: power of 1024 x 32768 340 us; two arrays at 131072
+        return (double)p->N * (both ? 13.5 : 10.0);
+    if (!p->mr) {
+        const int L = p->M <= kMaxFft ? p->M : p->N;  // clusters transform all N points
+        const double ps = L <= 256 ? 2.7 : L <= 4096 ? 3.1 : L <= 8192 ? 4.0 : L <= kMaxFft ? 5.0
+                          : L <= 32768 ? 6.0 : L <= 65536 ? 7.1 : 9.5;
+        // a folded row's first pass sums fold bins per point: 4096 / 4 3.4 ... 6.5, 16384 / 4 3.9 ... 6.5
+        return (double)L * ((both ? 1.15 : 1.0) * ps + (L < p->N ? 1.5 : 0.0));
+    }
+    double ps;
+    if (p->cl > 1)  // one kernel for two local rows per SM: 20000 5.7, 60000 8.4; 16464 12.7, 6.3 compiled for it
+        ps = p->sch.fixed_cl >= 0 ? 6.2 : compiled ? 7.0 : 12.5;
+    else  // 3000 4.3, 10000 4.0; 6400 5.2, 3200 6.3; 2304 8.1, 6300 9.4; compiled for the plan 2.9 ... 6.2
+        ps = p->sch.fixed >= 0 ? 4.1 : compiled ? 4.7 : p->sch.fast >= 0 ? 5.7 : 8.6;
+    return (double)p->N * (both ? 1.1 : 1.0) * ps;
 }
 
 }  // namespace
@@ -489,17 +526,22 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     std::vector<int4> list;
     std::vector<int> rest;
     ZoomShape sh;
-    sh.N = p->N;
     sh.M = M;
     sh.sub = p->d / f;
     sh.n_out = p->n_out;
-    sh.rest_cost = row_cost(p);
+    sh.both = (p->outputs & (p->outputs - 1)) != 0;
+    // a compiled plan starts from the split of one that is not, so that its results
+    // are the same bits as far as the same scales stay on classes
+    sh.rest_cost = row_cost(p, sh.both, false);
+    sh.compiled_cost = p->compiled ? row_cost(p, sh.both, true) : 0.0;
     sh.phase = (p->outputs & CWT_OUT_PHASE) != 0;
     sh.rows_only = false;
     sh.wide = true;
-    sh.channels = 64;
-    sh.row_bytes = (double)p->n_out * (((p->outputs & CWT_OUT_COMPLEX) ? 8 : 0) + ((p->outputs & CWT_OUT_POWER) ? 4 : 0) +
-                                       ((p->outputs & CWT_OUT_PHASE) ? 4 : 0));
+    // between plans of a few channels, which would take launches that pay only
+    // beyond them, and large ones, which want each scale on its cheapest form
+    // (16384 x 100 at 64 channels: 272 us decided at 64, 258 at 32, 264 at 8; 2500 x
+    // 100: 64, 64, 72; 2 x 30000: 48, 48, 37)
+    sh.channels = 40;
     zoom_select(sh, S, band.data(), &classes, &list, &rest);
     // columns and grids stay within 31 bits
     for (const ZoomClass &c : classes)

@@ -49,16 +49,17 @@ struct ZoomClass {
     int wide;  // -1: not wide
 };
 
-// What zoom_select decides from: a row of N bins on M points of which every
-// sub-th is kept, output rows of n_out samples (0: of any length), the cost of
-// a row (ps) on the kernels that take the rest, and whether the phase is asked
-// for.
+// What zoom_select decides from: a row on M points of which every sub-th is kept,
+// output rows of n_out samples (0: of any length), the cost of a row (ps) on the
+// kernels that take the rest and, if that is on kernels compiled for the plan, its
+// cost there (else 0), and whether the phase, and whether more than one output
+// array, is asked for.
 struct ZoomShape {
-    int N, M, sub, n_out;
-    double rest_cost;
-    bool phase, rows_only, wide;  // only zoom_row_kernel; zoom_wide.cuh allowed
-    double channels;   // nominal, for the cost of a launch against that of its rows
-    double row_bytes;  // output bytes of one row
+    int M, sub, n_out;
+    double rest_cost, compiled_cost;
+    bool phase, both;
+    bool rows_only, wide;  // only zoom_row_kernel; zoom_wide.cuh allowed
+    double channels;  // nominal, for the cost of a launch against that of its rows
 };
 
 // Splits S scales with bands band[2 s] (start), band[2 s + 1] (length) into
