@@ -119,6 +119,7 @@ const void *wide_kernel_of(int i, int mode) {
 }
 
 constexpr int kMaxSmem = 227 * 1024;
+constexpr int kSms = 152;
 
 // Rows that P consecutive columns, the first a multiple of P, can meet.
 int rows_met(int P, int R) {
@@ -141,13 +142,14 @@ int row_stride(int i, int nr, int R) {
     return R < 16 && nr > 1 ? len + ((R - len) & 15) : len;
 }
 
-// Rows per CTA of zoom_row_kernel: the most threads at work on a tile of about
-// 5000 points (several CTAs per SM), up to 8400.
-int rows_per_cta(int i, int M, int R) {
+// Rows per CTA of zoom_row_kernel for a launch of `rows`: the most threads at work
+// on a tile of about 5000 points (several CTAs per SM), up to 8400; few enough
+// that two CTAs per SM have rows.  A row's arithmetic does not depend on it.
+int rows_per_cta(int i, int M, int R, long long rows) {
     const int T = inst(i).T;
     int best = 1;
     double score = -1;
-    for (int nr = 1; nr * R <= T && (nr == 1 || nr * M <= 8400); ++nr) {
+    for (int nr = 1; nr * R <= T && (nr == 1 || (nr * M <= 8400 && (long long)nr * 2 * kSms <= rows)); ++nr) {
         const int C = nr * R;
         double v = (double)(T / C * C) / T;
         if (nr * M < 4000) v *= nr * M / 4000.0;
@@ -155,6 +157,15 @@ int rows_per_cta(int i, int M, int R) {
         if (v > score) score = v, best = nr;
     }
     return best;
+}
+
+// Whether rows of M points, R residues, can run on instance i by whole rows (MODE
+// 2, not for the phase), for any number of rows in a launch.
+bool row_fits(int i, int M, int R) {
+    if (R < 2 || R > inst(i).T || M > (inst(i).T > 128 ? kZoomRowPoints : 5632)) return false;
+    for (int nr = rows_per_cta(i, M, R, 1ll << 40); nr >= 1; --nr)
+        if (row_smem_of(i, nr, row_stride(i, nr, R), R) > kMaxSmem) return false;
+    return true;
 }
 
 // Opt instance i (mode) into the largest shared memory, once per device.
@@ -264,8 +275,7 @@ void zoom_select(const ZoomShape &z, int S, const int *band, std::vector<ZoomCla
         // few residues leave a row's band product little use and its stores short
         if (!z.rows_only && (R >= 4 || inst(i).P <= 4) && smem_of(i, rows_met(inst(i).P, R)) <= kMaxSmem)
             all.push_back({2 * i, column_cost(i, z), cap});
-        if (!z.phase && R >= 2 && z.M <= (inst(i).T > 128 ? kZoomRowPoints : 5632) && R <= inst(i).T &&
-            row_smem_of(i, rows_per_cta(i, z.M, R), row_stride(i, rows_per_cta(i, z.M, R), R), R) <= kMaxSmem)
+        if (!z.phase && row_fits(i, z.M, R))
             all.push_back({2 * i + 1, whole_cost(i, z), cap});
     }
     if (z.wide)
@@ -369,7 +379,15 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     a.magL = zoom_magic((unsigned)a.L);
     a.magR = zoom_magic((unsigned)R);
     a.magNs = zoom_magic((unsigned)c.ns);
-    const int mode = c.rows ? 2 : a.oph || a.sub != 1 ? 1 : 0;
+    // A column group that meets several rows forms their band products one after the
+    // other, a load latency each, which a launch too small to fill the GPU does not
+    // hide: such launches run by whole rows, the same arithmetic on the same tables
+    // (16 x 32, 88 rows of 4096 points 6.4 us by columns, 3.9 by rows; 352 rows 9.0
+    // and 6.3; 32 columns that meet two rows: 5.4 and 5.7 at 312).
+    const int met = rows_met(t.P, R);
+    const bool small = (double)rows * a.M <= (t.P <= 16 && met == 2 ? 1.5e6 : 5e5) && met >= (t.P >= 32 ? 3 : 2);
+    const bool by_rows = c.rows || (small && !a.oph && row_fits(c.inst, a.M, R));
+    const int mode = by_rows ? 2 : a.oph || a.sub != 1 ? 1 : 0;
     cudaError_t e = ensure_zoom_smem(c.inst, mode);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr;
@@ -380,8 +398,8 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (c.rows) {
-        a.nr = rows_per_cta(c.inst, a.M, R);
+    if (by_rows) {
+        a.nr = rows_per_cta(c.inst, a.M, R, rows);
         a.nrows = (int)rows;
         a.ps = position_stride(c.inst, a.nr, R);
         a.rs = row_stride(c.inst, a.nr, R);

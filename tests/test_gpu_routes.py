@@ -1,6 +1,10 @@
-"""Which transform each scale takes (cwt_plan_routes)."""
+"""Which transform each scale takes (cwt_plan_routes), and that a channel's bits
+depend neither on how many channels run beside it nor on the form that a launch
+of few rows takes."""
 import numpy as np
 import pytest
+
+from eeg_synth import eeg
 
 pytestmark = pytest.mark.gpu
 
@@ -44,3 +48,33 @@ def test_compiled_rows_take_the_scales_that_classes_run_slower(lib):
 def test_most_scales_of_everyday_plans_run_by_classes(lib):
     whole, one, two = _routes(lib, 10000, 100, 1, 100, outputs=("complex", "power"), pad="smooth")
     assert one + two >= 70 and whole + one + two == 100
+
+
+# samples, scales, outputs, decimation, padding: launches of few rows take another
+# form than those of many (column groups that meet two, four and more rows, whole
+# rows by one and by several per CTA)
+SHAPES = [
+    (4000, 100, ("complex", "power"), 1, "pow2"), (700, 40, ("power",), 1, "pow2"), (1500, 60, ("complex",), 2, "pow2"),
+    (3000, 60, ("power",), 4, "smooth"), (2500, 60, ("power",), 1, "smooth"), (3001, 61, ("complex", "power"), 1, "smooth"),
+    (8000, 60, ("power",), 3, "pow2"), (394, 40, ("power",), 1, "smooth"), (9000, 20, ("complex", "power"), 1, "smooth"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(SHAPES)))
+def test_bits_of_a_channel_do_not_depend_on_the_others(lib, case):
+    import torch
+    n, S, outs, d, pad = SHAPES[case]
+    C, lo = 48, max(2.0, 3000.0 / n)
+    x = torch.from_numpy(eeg(2800 + case, C, n, 1000.0, np.float32)).cuda()
+    args = (1000.0, np.geomspace(lo, 90, S), np.linspace(3, 10, S))
+    kw = dict(outputs=outs, decimation=d, pad=pad)
+    whole = lib.CWT(C, n, *args, **kw)
+    ref = whole(x)
+    for c0, c1 in ((0, 1), (7, 9), (20, 28), (47, 48)):
+        part = lib.CWT(c1 - c0, n, *args, **kw)
+        out = part(x[c0:c1].clone())  # aligned
+        torch.cuda.synchronize()
+        for k in outs:
+            assert torch.equal(out[k], ref[k][c0:c1]), (k, c0)
+        part.close()
+    whole.close()
