@@ -99,16 +99,18 @@ cwt_status check_after(cwt_plan_s *p, cudaStream_t st) {
     return CWT_OK;
 }
 
-// The scale blocks in slices of `slice` channels, done(c0, k) after the kernels
-// of channels [c0, c0 + k) are in the stream.
+// The scale blocks in slices of channels, `first` of them and then four times as
+// many each time, done(c0, k) after the kernels of channels [c0, c0 + k) are in
+// the stream.
 template <typename Done>
-cudaError_t scale_blocks_sliced(const cwt_plan_s *p, void *oc, void *op, void *oph, cudaStream_t st, int slice,
+cudaError_t scale_blocks_sliced(const cwt_plan_s *p, void *oc, void *op, void *oph, cudaStream_t st, int first,
                                 const Done &done) {
     try {
         cwt_plan_s q = *p;  // the same plan over some of the channels
         cudaError_t e = cudaSuccess;
-        for (int c0 = 0; c0 < p->C && e == cudaSuccess; c0 += slice) {
-            q.C = std::min(slice, p->C - c0);
+        long long slice = first;
+        for (int c0 = 0; c0 < p->C && e == cudaSuccess; c0 += q.C, slice *= 4) {
+            q.C = (int)std::min<long long>(slice, p->C - c0);
             q.spec = p->spec + (size_t)c0 * (size_t)p->N;
             if (p->tc_chmax) q.tc_chmax = p->tc_chmax + c0;
             const size_t at = out_elem_bytes(p) * (size_t)c0 * (size_t)p->S * (size_t)p->n_out;
@@ -127,7 +129,7 @@ struct NoSlices {
 
 template <typename Done = NoSlices>
 cwt_status run_execute(cwt_plan_s *p, const void *sig, void *oc, void *op, void *oph, cudaStream_t st,
-                       int slice = 0, const Done &done = Done()) {
+                       int first_slice = 0, const Done &done = Done()) {
     cwtk::ProfEvent ev{};
     cudaError_t e = prof_begin(p, CWT_KERNEL_FORWARD_FFT, st, &ev);
     if (e == cudaSuccess) e = cwtk::launch_forward(p, sig, st);
@@ -136,7 +138,8 @@ cwt_status run_execute(cwt_plan_s *p, const void *sig, void *oc, void *op, void 
     if (e == cudaSuccess) e = prof_end(p, st, &ev);
     if (e == cudaSuccess) e = prof_begin(p, CWT_KERNEL_SCALE_BLOCK, st, &ev);
     if (e == cudaSuccess)
-        e = slice ? scale_blocks_sliced(p, oc, op, oph, st, slice, done) : cwtk::launch_scale_block(p, oc, op, oph, st);
+        e = first_slice ? scale_blocks_sliced(p, oc, op, oph, st, first_slice, done)
+                        : cwtk::launch_scale_block(p, oc, op, oph, st);
     if (e == cudaSuccess) e = prof_end(p, st, &ev);
     if (e != cudaSuccess) return fail_cuda(p, e);
     return check_after(p, st);
@@ -580,19 +583,22 @@ cwt_status cwt_execute_host(cwt_plan p, const void *h_signal, void *h_complex, v
     void *mp = wp ? mapped_host_ptr(h_power) : nullptr;
     void *mph = wph ? mapped_host_ptr(h_phase) : nullptr;
     // Residue classes store runs of a few outputs, which fill the link less well
-    // than a copy does (64 x 10000 x 100, 768 MB: 4.38 ms written directly, 4.12 in
-    // slices of channels copied while the next are computed, 4.30 in slices of 20
-    // MB); whole rows and small outputs are written directly.
-    constexpr size_t kSliceBytes = (size_t)48 << 20;
+    // than a copy does: their outputs are staged, and slices of channels copied
+    // while the next are computed, which takes a twentieth to a quarter of the time:
+    // a small first slice starts the link early, and few large ones follow, because
+    // each copy leaves it idle for about 4 us.  Outputs up to 6 MB are written directly.
+    // (64 x 10000 x 100, 768 MB: 4.38 ms written directly, 4.05 in slices, 4.09 as
+    // whole rows written directly; 8 x 10000 x 100, 32 MB: 240, 217 and 209 us.)
+    constexpr size_t kDirectBytes = (size_t)6 << 20, kFirstBytes = (size_t)2 << 20;
     const size_t mapped = (mc ? 2 * out_b : 0) + (mp ? out_b : 0) + (mph ? out_b : 0);
-    if (p->zoom && mapped > kSliceBytes) {
+    if (p->zoom && mapped > kDirectBytes) {
         if (!p->copy_stream) e = cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking);
         if (e == cudaSuccess && !p->sliced) e = cudaEventCreateWithFlags(&p->sliced, cudaEventDisableTiming);
         if (e != cudaSuccess) return fail_cuda(p, e);
         const size_t ch_b = out_b / (size_t)p->C;
-        const int slice = (int)std::max<size_t>(1, (size_t)p->C / (mapped / kSliceBytes + 1));
+        const int first = (int)std::max<size_t>(1, kFirstBytes / (mapped / (size_t)p->C));
         const cwt_status s = run_execute(
-            p, p->stage_in, p->stage_c, p->stage_p, p->stage_ph, st, slice, [&](int c0, int k) -> cudaError_t {
+            p, p->stage_in, p->stage_c, p->stage_p, p->stage_ph, st, first, [&](int c0, int k) -> cudaError_t {
                 cudaError_t r = cudaEventRecord(p->sliced, st);
                 if (r == cudaSuccess) r = cudaStreamWaitEvent(p->copy_stream, p->sliced, 0);
                 auto copy = [&](void *h, void *d, size_t b) {
