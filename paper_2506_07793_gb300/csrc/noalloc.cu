@@ -52,8 +52,14 @@ struct NaScales {
 };
 
 // Exponent of the larger of Eq. 3's two terms at u = nu / F (the second is the
-// admissibility term, kappa = exp(-sigma^2 / 2)).
-__device__ __forceinline__ float na_exponent(float u, float h) { return -h * (u * u + 1.f - 2.f * fmaxf(u, 0.f)); }
+// admissibility term, kappa = exp(-sigma^2 / 2)).  Squared after the difference:
+// u^2 + 1 - 2 u is off by 1e-7, which h = sigma^2 / 2 makes more than the cut below
+// from sigma = 30000 up (bins beside the carrier were lost); this form by 2 h |u - 1|
+// 1e-7, below 1 wherever two bins of 16384 compare.
+__device__ __forceinline__ float na_exponent(float u, float h) {
+    const float d = u - 1.f;
+    return u > 0.f ? -h * d * d : -h * (u * u + 1.f);
+}
 
 // Eq. 3 (Morlet spectrum in Hz) in FP64 summed over aliases, in the plan
 // generator's order.  Terms e^40 below the bin's largest (exponent `top`) are
