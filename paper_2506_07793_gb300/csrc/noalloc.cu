@@ -337,11 +337,12 @@ extern "C" cwt_status cwt_execute_noalloc(const float *d_signal, int channels, i
         return CWT_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     char *base = nullptr;
-    cudaError_t e = na_setup(dev, st, &base);
-    // not inside a stream capture (see cwt.h), whether or not anything is copied
+    // not inside a stream capture (see cwt.h), whether or not anything is copied;
+    // asked before the set-up, whose launch and wait would invalidate the capture
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
     if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return CWT_ECUDA;
+    if (e == cudaSuccess) e = na_setup(dev, st, &base);
     NaScales inl;
     const double *par = nullptr;
     if (n_freqs <= kNaInline) {
