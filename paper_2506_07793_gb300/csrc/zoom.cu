@@ -368,7 +368,6 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     const ZoomInst &t = inst(c.inst);
     const int R = a.M / t.Q;
     const long long rows = chans * c.ns;
-    if (rows >= 2147483647ll || rows * R >= 2147483647ll) return cudaErrorInvalidValue;
     a.R = R;
     a.L = R * t.QA;
     a.twl = twl;
@@ -387,6 +386,8 @@ cudaError_t zoom_launch(const ZoomClass &c, ZoomArgs a, long long chans, const f
     const int met = rows_met(t.P, R);
     const bool small = (double)rows * a.M <= (t.P <= 16 && met == 2 ? 1.5e6 : 5e5) && met >= (t.P >= 32 ? 3 : 2);
     const bool by_rows = c.rows || (small && !a.oph && row_fits(c.inst, a.M, R));
+    // the kernels count rows, and columns those of all rows, in 31 bits
+    if ((by_rows ? rows : rows * R) >= 2147483647ll) return cudaErrorInvalidValue;
     const int mode = by_rows ? 2 : a.oph || a.sub != 1 ? 1 : 0;
     cudaError_t e = ensure_zoom_smem(c.inst, mode);
     if (e != cudaSuccess) return e;
