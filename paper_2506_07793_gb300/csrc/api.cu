@@ -390,7 +390,6 @@ cwt_status cwt_plan_create(cwt_plan *out, int channels, int samples, double fs,
     }
     p->compiled = p->jit || tune;
     if (e == cudaSuccess) e = cwtk::launch_bank(p, st);
-    if (e == cudaSuccess) e = cwtk::zoom_plan_create(p, st);
     if (e == cudaSuccess && tc) {
         e = cwtk::dmalloc(&p->tc_chmax, sizeof(float) * (size_t)channels);
         if (e == cudaSuccess) e = cwtk::dmalloc(&p->tc_wl1, sizeof(float) * (size_t)n_freqs);
@@ -398,6 +397,7 @@ cwt_status cwt_plan_create(cwt_plan *out, int channels, int samples, double fs,
         if (e == cudaSuccess) e = cwtk::launch_tc_wl1(p, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
+    if (e == cudaSuccess) e = cwtk::zoom_plan_create(p, st);
     if (e == cudaSuccess && tune) {
         // candidates timed on the plan's rows once the bank is in place; a
         // failure leaves the plan on the runtime-schedule kernels
@@ -465,7 +465,7 @@ cwt_status cwt_plan_info(cwt_plan p, cwt_plan_info_t *info) {
     info->device = p->device;
     info->io_dtype = p->io;
     info->output_kinds = p->outputs;
-    info->workspace_bytes = p->bytes + p->stage_bytes;
+    info->workspace_bytes = cwt_plan_workspace_bytes(p);
     info->bank_ms = p->bank_ms;
     info->precision = p->precision;
     info->cluster = p->mr ? p->cl : (p->M > cwtk::kMaxFft ? p->M / cwtk::kMaxFft : 1);
@@ -512,7 +512,9 @@ cwt_status cwt_smooth_cluster(int n_fft, int specialize, int *cluster, int *radi
     return CWT_OK;
 }
 
-size_t cwt_plan_workspace_bytes(cwt_plan p) { return p ? p->bytes + p->stage_bytes : 0; }
+size_t cwt_plan_workspace_bytes(cwt_plan p) {
+    return p ? p->bytes + p->stage_bytes + cwtk::batch_bytes(p->batch) : 0;
+}
 
 const char *cwt_plan_last_error(cwt_plan p) { return p ? p->last_error.c_str() : ""; }
 

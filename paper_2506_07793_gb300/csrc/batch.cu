@@ -108,6 +108,11 @@ void free_batch_state(BatchState *b) {
     delete b;
 }
 
+size_t batch_bytes(const BatchState *b) {
+    if (!b) return 0;
+    return b->bytes + b->items_cap * sizeof(BatchItem) + b->eps_cap * sizeof(ZoomEpoch) + b->ws_cap * sizeof(float2);
+}
+
 namespace {
 
 template <int RI>
@@ -255,8 +260,10 @@ int epoch_log2(const cwt_plan_s *p, const cwt_epoch &ep) {
     return ilog2c(N);
 }
 
-// Items, chunks and epoch tables of a new shape, uploaded.
-cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, int n_epochs, cudaStream_t st) {
+// Items, chunks of up to *ws_bytes (or one epoch) of workspace and epoch tables of a
+// new shape, uploaded; *ws_bytes becomes the largest chunk's.
+cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, int n_epochs, size_t *ws_bytes,
+                       cudaStream_t st) {
     const int C = p->C, S = p->S, d = p->d;
     std::vector<BatchItem> items;
     std::vector<ZoomEpoch> eps;
@@ -268,9 +275,9 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
         BatchChunk ch;
         ch.item0 = items.size();
         int last = first;
-        for (; last < n_epochs; ++last) {  // at least one epoch, then up to kWsBytes
+        for (; last < n_epochs; ++last) {
             const size_t w = (size_t)C * (size_t)b->len[epoch_log2(p, epochs[last])].wn;
-            if (last > first && (ch.ws + w) * sizeof(float2) > kWsBytes) break;
+            if (last > first && (ch.ws + w) * sizeof(float2) > *ws_bytes) break;
             ch.ws += w;
         }
         size_t ws = 0;
@@ -304,6 +311,7 @@ cudaError_t make_shape(cwt_plan_s *p, BatchState *b, const cwt_epoch *epochs, in
         chunks.push_back(ch);
         first = last;
     }
+    *ws_bytes = ws_max * sizeof(float2);
     cudaError_t e = grow(&b->d_items, &b->items_cap, std::max<size_t>(items.size(), 1));
     if (e == cudaSuccess) e = grow(&b->d_eps, &b->eps_cap, eps.size());
     if (e == cudaSuccess) e = grow(&b->d_ws, &b->ws_cap, ws_max);
@@ -343,7 +351,15 @@ cudaError_t batch_prepare(cwt_plan_s *p, const cwt_epoch *epochs, int n_epochs, 
                       std::equal(b->shape.begin(), b->shape.end(), epochs, [](const cwt_epoch &x, const cwt_epoch &y) {
                           return x.in_offset == y.in_offset && x.out_offset == y.out_offset && x.samples == y.samples;
                       });
-    return same ? cudaSuccess : make_shape(p, b, epochs, n_epochs, st);
+    if (same) return cudaSuccess;
+    // more and smaller chunks where memory is short: slower, the same values
+    size_t ws = kWsBytes, tried = (size_t)-1;
+    while ((e = make_shape(p, b, epochs, n_epochs, &ws, st)) == cudaErrorMemoryAllocation && ws < tried) {
+        cudaGetLastError();  // clear the non-sticky error
+        tried = ws;
+        ws /= 4;
+    }
+    return e;
 }
 
 cudaError_t batch_run(cwt_plan_s *p, const float *in, float2 *oc, float *op, float *oph, cudaStream_t st) {

@@ -58,6 +58,7 @@ void zoom_routes(const ZoomPlan *z, int *classes, int *two_kernels);  // scales 
 
 struct BatchState;
 void free_batch_state(BatchState *b);
+size_t batch_bytes(const BatchState *b);  // device bytes: banks, items, workspace
 
 struct ProfEvent {
     int kernel;

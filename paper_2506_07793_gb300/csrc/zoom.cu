@@ -590,14 +590,21 @@ static cudaError_t zoom_plan_build(cwt_plan_s *p, cudaStream_t st) {
     for (const ZoomClass &c : classes)
         if (c.wide >= 0) wide_rows = std::max(wide_rows, (long long)p->C * c.ns);
     wide_rows = std::min(wide_rows, (long long)std::max<size_t>(1, kWideBytes / (sizeof(float2) * (size_t)M)));
-    z->wide_rows = (int)wide_rows;
-    if (e == cudaSuccess && wide_rows) e = dmalloc(&z->d_wide, 2 * sizeof(float2) * (size_t)M * (size_t)wide_rows);
     if (e == cudaSuccess && !rest.empty()) {
         e = dmalloc(&p->rest_list, sizeof(int) * rest.size());
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(p->rest_list, rest.data(), sizeof(int) * rest.size(), cudaMemcpyHostToDevice, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // fewer rows at a time where memory is short: slower, the same values
+    while (e == cudaSuccess && wide_rows) {
+        e = dmalloc(&z->d_wide, 2 * sizeof(float2) * (size_t)M * (size_t)wide_rows);
+        if (e != cudaErrorMemoryAllocation || wide_rows == 1) break;
+        cudaGetLastError();  // clear the non-sticky error
+        e = cudaSuccess;
+        wide_rows = std::max(1ll, wide_rows / 4);
+    }
+    z->wide_rows = (int)wide_rows;
     p->rest_scales = (int)rest.size();
     p->bytes += sizeof(int4) * list.size() + sizeof(int) * rest.size() + (p->mr ? sizeof(float2) * total_l : 0) +
                 2 * sizeof(float2) * (size_t)M * (size_t)wide_rows;
