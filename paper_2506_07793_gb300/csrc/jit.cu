@@ -456,63 +456,35 @@ JitKernels *jit_tune(cwt_plan_s *p, cudaStream_t st, std::string *log) {
         k[i] = jit_kernels(cand[i], rows[i], cl, p->device, &lg);
         if (!k[i] && log->empty()) *log = lg;
     }
-    // time each on the plan's own rows (all of them, or as many as 256 MB of
-    // scratch outputs hold)
+    // time each on what the plan will run on it: the forward FFTs and the scales that
+    // are not run by residue classes, over all channels or as many as 256 MB of
+    // scratch outputs hold
     const size_t esz = p->io == CWT_DTYPE_F64 ? 8 : 4;
     const size_t row_bytes = (size_t)p->n_out * esz *
                              (((p->outputs & CWT_OUT_COMPLEX) ? 2 : 0) + ((p->outputs & CWT_OUT_POWER) ? 1 : 0) +
                               ((p->outputs & CWT_OUT_PHASE) ? 1 : 0));
-    const size_t cap = row_bytes ? ((size_t)256 << 20) / row_bytes : (size_t)total;
-    const int trows = (int)std::max<size_t>(1, std::min<size_t>((size_t)total, cap));
-    const size_t cells = (size_t)trows * (size_t)p->n_out;
-    void *oc = nullptr, *op = nullptr, *oph = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (p->outputs & CWT_OUT_COMPLEX) e = dmalloc(&oc, cells * 2 * esz);
-    if (e == cudaSuccess && (p->outputs & CWT_OUT_POWER)) e = dmalloc(&op, cells * esz);
-    if (e == cudaSuccess && (p->outputs & CWT_OUT_PHASE)) e = dmalloc(&oph, cells * esz);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->spec, 0, sizeof(float2) * (size_t)p->C * p->N, st);
+    const int chans = (int)std::max<size_t>(
+        1, std::min<size_t>((size_t)p->C, ((size_t)256 << 20) / (row_bytes * (size_t)p->S)));
+    const size_t cells = p->rest_scales ? (size_t)chans * (size_t)p->S * (size_t)p->n_out : 0;
+    const size_t in_b = (size_t)chans * (size_t)p->n * esz;
+    void *x = nullptr, *oc = nullptr, *op = nullptr, *oph = nullptr;
+    cudaError_t e = dmalloc(&x, in_b);
+    if (e == cudaSuccess) e = cudaMemsetAsync(x, 0, in_b, st);
+    if (e == cudaSuccess && cells && (p->outputs & CWT_OUT_COMPLEX)) e = dmalloc(&oc, cells * 2 * esz);
+    if (e == cudaSuccess && cells && (p->outputs & CWT_OUT_POWER)) e = dmalloc(&op, cells * esz);
+    if (e == cudaSuccess && cells && (p->outputs & CWT_OUT_PHASE)) e = dmalloc(&oph, cells * esz);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    MrArgs a;  // one-CTA rows
-    a.spec = p->spec;
-    a.bank = p->bank;
-    a.band = p->band;
-    a.twN = p->twN;
-    a.out_c = oc;
-    a.out_p = op;
-    a.out_ph = oph;
-    a.list = nullptr;
-    a.S = a.ns = p->S;
-    a.n_out = p->n_out;
-    a.sub = p->d;
-    a.total_rows = trows;
-    a.f64 = p->io == CWT_DTYPE_F64;
-    ClMrArgs ca;  // cluster rows: the first trows rows (the grid is trows clusters)
-    ca.spec = p->spec;
-    ca.bank = p->bank;
-    ca.band = p->band;
-    ca.twL = p->twL;
-    ca.twN = p->twN;
-    ca.out_c = oc;
-    ca.out_p = op;
-    ca.out_ph = oph;
-    ca.list = nullptr;
-    ca.S = ca.ns = p->S;
-    ca.n_out = p->n_out;
-    ca.sub = p->d;
-    ca.f64 = p->io == CWT_DTYPE_F64;
     const bool compiled_in = cl == 1 ? p->sch.fixed >= 0 : p->sch.fixed_cl >= 0;
+    cwt_plan_s q = *p;  // the plan over some channels, on a candidate
+    q.C = chans;
     auto launch = [&](int i) -> cudaError_t {
-        if (cl == 1) return i >= 0 ? sb_launch_k(k[i], a, st) : mr_fixed_sb_launch(p, a, st);
-        const JitKernels *kk = i >= 0 ? k[i] : nullptr;
-        if (!kk) return cl_mr_fixed_sb(p, ca, st, trows);
-        ClMrArgs args = ca;
-        MrSchedule sch = cand[i];
-        void *params[] = {&args, &sch};
-        const CUresult r = driver().launch_kernel(kk->sb, (unsigned)(trows * cl), 1, 1, (unsigned)kk->threads, 1,
-                                                  1, (unsigned)kk->smem, (CUstream)st, params, nullptr);
-        return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
+        q.jit = i >= 0 ? k[i] : nullptr;
+        q.sch = i >= 0 ? cand[i] : p->sch;
+        cudaError_t r = launch_forward(&q, x, st);
+        if (r == cudaSuccess && q.rest_scales) r = launch_scale_block_mr(&q, oc, op, oph, st);
+        return r;
     };
     // candidate -1: the length's compiled-in kernel, when it has one
     int best = -2;
@@ -537,6 +509,7 @@ JitKernels *jit_tune(cwt_plan_s *p, cudaStream_t st, std::string *log) {
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
+    cudaFree(x);
     cudaFree(oc);
     cudaFree(op);
     cudaFree(oph);

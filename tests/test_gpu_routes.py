@@ -45,6 +45,26 @@ def test_compiled_rows_take_the_scales_that_classes_run_slower(lib):
     assert _routes(lib, 6300, 60, 2, 40, specialize=1, **kw)[1] >= 50
 
 
+@pytest.mark.parametrize("n,lo,hi", [(6300, 2, 40), (6300, 2, 400), (16464, 1, 60)])
+def test_tuning_runs_what_the_plan_runs(lib, n, lo, hi):
+    """specialize = 2 times the forward FFTs and the scales left to whole rows, which
+    may be none: no scratch for outputs that nothing writes, and the oracle's values."""
+    import oracle
+    import torch
+    from tests.metrics import FP32_TOL, power_err
+    S, C = 6, 3
+    f, c = np.geomspace(lo, hi, S), np.linspace(3, 10, S)
+    x = eeg(2790 + hi, C, n, 1000.0, np.float32)
+    t = lib.CWT(C, n, 1000.0, f, c, pad="smooth", specialize=2)
+    try:
+        assert t.info.specialized in (0, 2) and t.info.fixed_kernel == 1
+        out = t(torch.from_numpy(x).cuda())["power"].cpu().numpy()
+        ref = oracle.cwt(x.astype(np.float64), t.info.fft_length, 1000.0, f, c)
+        assert power_err(out, ref).max() <= FP32_TOL
+    finally:
+        t.close()
+
+
 def test_most_scales_of_everyday_plans_run_by_classes(lib):
     whole, one, two = _routes(lib, 10000, 100, 1, 100, outputs=("complex", "power"), pad="smooth")
     assert one + two >= 70 and whole + one + two == 100
