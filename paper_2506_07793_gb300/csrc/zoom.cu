@@ -162,7 +162,7 @@ int rows_per_cta(int i, int M, int R, long long rows) {
 // Whether rows of M points, R residues, can run on instance i by whole rows (MODE
 // 2, not for the phase), for any number of rows in a launch.
 bool row_fits(int i, int M, int R) {
-    if (R < 2 || R > inst(i).T || M > (inst(i).T > 128 ? kZoomRowPoints : 5632)) return false;
+    if (R < 2 || R > inst(i).T || M > zoom_row_points(inst(i).T)) return false;
     for (int nr = rows_per_cta(i, M, R, 1ll << 40); nr >= 1; --nr)
         if (row_smem_of(i, nr, row_stride(i, nr, R), R) > kMaxSmem) return false;
     return true;
@@ -481,8 +481,8 @@ cudaError_t wide_launch(const ZoomClass &c, const ZoomArgs &args, long long chan
 
 namespace {
 
-// Half the workspace of zoom_wide.cuh (32 x 122880 x 128 power: 1.80 ms with 28
-// MB, 1.69 with 40, 1.61 with 57, 1.67 with 80, 1.62 with 400).
+// Half the workspace of zoom_wide.cuh: enough that more gains nothing (32 x 122880
+// x 128 power: 1.80 ms with 28 MB, 1.69 with 40, then 1.61 ... 1.67 up to 400).
 constexpr size_t kWideBytes = (size_t)56 << 20;
 
 // Cost of one row (ps) on the whole-row kernels, for the bands that are left to

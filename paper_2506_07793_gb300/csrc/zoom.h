@@ -15,9 +15,17 @@
 namespace cwtk {
 
 // The kernel of instance I: zoom_kernel MODE 0 or 1, or (2) zoom_row_kernel
-// (zoom_inst_<g>.cu).
+// (zoom_inst_<g>.cu), null where its rows of two residues are too long for that.
 template <int I>
 const void *zoom_entry(int mode);
+
+// The longest rows that zoom_row_kernel holds on T threads.
+constexpr int zoom_row_points(int T) { return T > 128 ? kZoomRowPoints : 5632; }
+template <class Z>
+const void *zoom_row_entry() {
+    if constexpr (2 * Z::Q <= zoom_row_points(Z::T)) return (const void *)&zoom_row_kernel<Z>;
+    else return nullptr;
+}
 
 #define CWT_ZOOM_DEFINE(I, QA, QB, QC, P, T, MINB, COST)                        \
     template <>                                                                 \
@@ -25,7 +33,7 @@ const void *zoom_entry(int mode);
         using Z = ZoomCfg<QA, QB, QC, P, T, MINB>;                              \
         return mode == 0   ? (const void *)&zoom_kernel<Z, 0>                   \
                : mode == 1 ? (const void *)&zoom_kernel<Z, 1>                   \
-                           : (const void *)&zoom_row_kernel<Z>;                 \
+                           : zoom_row_entry<Z>();                               \
     }
 
 // The kernels of zoom_wide.cuh: first radix i, remaining length I in MODE 0 or 1.
