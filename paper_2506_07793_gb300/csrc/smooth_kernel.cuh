@@ -43,11 +43,9 @@ cudaError_t mr_sb_launch(const cwt_plan_s *p, const MrArgs &a, cudaStream_t st) 
     const int smem = rows * (p->N + (p->N >> 4)) * 8;
     const int threads = (rows * p->sch.T + 31) & ~31;
     const int grid = (a.total_rows + rows - 1) / rows;
-    // Double rows start after the forward FFTs: 106 x 93 x 120 points take 26.6
-    // us, 28.7 overlapped; float rows overlap (26 x 113 x 1845: 49.2, 51.3).
-    if (!a.f64) return launch_dependent(mr_scale_block_kernel<RA, RB>, grid, threads, smem, st, a, p->sch, rows);
-    mr_scale_block_kernel<RA, RB><<<grid, threads, smem, st>>>(a, p->sch, rows);
-    return cudaGetLastError();
+    // overlaps the end of the forward FFTs (double I/O: 106 x 93 x 120 22.6 -> 20.6 us,
+    // 26 x 1845 x 113 76.0 -> 74.2, 1 x 250 x 30 16.5 -> 12.5; never slower on ten shapes)
+    return launch_dependent(mr_scale_block_kernel<RA, RB>, grid, threads, smem, st, a, p->sch, rows);
 }
 
 // Forward FFT of each zero-padded channel (float32 or float64 samples), Eq. 2;
