@@ -51,16 +51,6 @@ struct NaScales {
     double F[kNaInline], sig[kNaInline];
 };
 
-// Exponent of the larger of Eq. 3's two terms at u = nu / F (the second is the
-// admissibility term, kappa = exp(-sigma^2 / 2)).  Squared after the difference:
-// u^2 + 1 - 2 u is off by 1e-7, which h = sigma^2 / 2 makes more than the cut below
-// from sigma = 30000 up (bins beside the carrier were lost); this form by 2 h |u - 1|
-// 1e-7, below 1 wherever two bins of 16384 compare.
-__device__ __forceinline__ float na_exponent(float u, float h) {
-    const float d = u - 1.f;
-    return u > 0.f ? -h * d * d : -h * (u * u + 1.f);
-}
-
 // Eq. 3 (Morlet spectrum in Hz) in FP64 summed over aliases, in the plan
 // generator's order.  Terms e^40 below the bin's largest (exponent `top`) are
 // left out: together they are under 1e-15 of it.
@@ -85,11 +75,11 @@ __device__ __forceinline__ double na_alias_sum(double base, double r, double lo,
 // band.  Bound by FP64 exponentials (the pipe retires a warp instruction in 16
 // cycles), so only bins whose exponent is within 27 of the scale's largest are
 // evaluated, once, and no other takes an FP64 instruction: the others are at
-// 2e-12 of the peak (a band's limit is 1e-10) and add under 1e-19 to the energy.  Where the peak itself comes out far
-// below its exponent (a carrier under the first bins, whose terms cancel) the
-// bound says nothing and every bin is evaluated.  40 scales at N = 2048: this
-// launch and the forward FFTs' in 9 us; two kernels that evaluated every bin
-// three times took 112 us.
+// 2e-12 of the peak (a band's limit is 1e-10) and add under 1e-19 to the energy.
+// Where the peak itself comes out far below its exponent (a carrier under the
+// first bins, whose terms cancel) the bound says nothing and every bin is
+// evaluated.  40 scales at N = 2048: 19 us, the forward FFTs beside it; two kernels
+// that evaluated every bin three times took 112.
 __global__ void __launch_bounds__(kNaThreads)
 na_bank_kernel(int N, int S, double fs, const double *par, const __grid_constant__ NaScales inl,
                float *__restrict__ bank, int *__restrict__ band) {
@@ -102,8 +92,15 @@ na_bank_kernel(int N, int S, double fs, const double *par, const __grid_constant
     const double hh = 0.5 * sg * sg, kappa = exp(-hh), r = fs / F, rN = 1.0 / (double)N;  // N is a power of two
     const double reach = 40.0 * F / sg, q_min = -reach / fs, q_max = (F + reach) / fs;
     const float h = (float)hh, du = (float)(r * rN), uN = (float)r;
-    auto exponent = [&](int k) {  // the nearest aliases of bin k: nu in [0, fs) and [-fs, 0)
-        return fmaxf(na_exponent((float)k * du, h), na_exponent((float)k * du - uN, h));
+    // The exponent of bin k's largest term: of its nearest aliases, u = nu / F in [0,
+    // fs / F) with exponent -h (u - 1)^2 and v = u - fs / F with that of the
+    // admissibility term, -h (v^2 + 1), kappa = exp(-h).  Squared after the difference:
+    // u^2 + 1 - 2 u is off by 1e-7, which h makes more than the cut below from sigma =
+    // 30000 up (bins beside the carrier were lost); this form by 2 h |u - 1| 1e-7, below
+    // 1 wherever two bins of 16384 compare.
+    auto exponent = [&](int k) {
+        const float u = (float)k * du, d = u - 1.f, v = u - uN;
+        return -h * fminf(d * d, v * v + 1.f);
     };
     __shared__ float sf[kNaThreads];
     float top = -INFINITY;
@@ -322,6 +319,7 @@ extern "C" cwt_status cwt_execute_noalloc(const float *d_signal, int channels, i
     if (!scales_on_grid(CWT_WAVELET_MORLET, freqs_hz, n_cycles, n_freqs, 3.0, fs, N)) return CWT_EINVAL;
     const int nblk = (N + kNaThreads - 1) / kNaThreads;
     const size_t off_par = align256(kTwBytes);
+    // (a region that nothing uses any more: the documented limit counts it)
     const size_t off_part = off_par + align256(sizeof(double) * 2 * (size_t)n_freqs);
     const size_t off_band = off_part + align256(sizeof(double) * (size_t)n_freqs * nblk);
     const size_t off_bank = off_band + align256(sizeof(int) * 2 * (size_t)n_freqs);
