@@ -161,8 +161,10 @@ typedef struct {
                        accumulation (the Cooley-Tukey factorisation of Section
                        "Fast Fourier transform"; error within 2e-3 of the row's
                        peak power): power-of-two N of 16384 ... 131072 only (else
-                       CWT_EUNSUPPORTED); not for cwt_execute_batch.  Scales whose
-                       band is narrow run in FP32, which is faster there */
+                       CWT_EUNSUPPORTED); not for cwt_execute_batch.  With float32
+                       I/O they only get the scales that FP32 residue classes do
+                       not run faster -- at most the widest bands, at most lengths
+                       none (cwt_plan_routes) -- unless whole_rows is 1 */
     int decimation; /* keep every d-th output sample, d >= 1 (default 1) */
     int pad_policy; /* cwt_pad_policy (default CWT_PAD_POW2) */
     int fft_length; /* 0: from pad_policy; else an explicit N >= samples that is a
@@ -228,7 +230,8 @@ typedef struct {
                                length of 15360, 15000 or 10000, e.g. N = 122880,
                                60000, 20000),
                                else 0; the forward FFTs then run on the same schedule */
-    int precision;          /* cwt_precision of the inverse FFTs */
+    int precision;          /* cwt_precision of the whole rows' inverse FFTs, as asked
+                               for (cwt_plan_routes: how many scales those are) */
     int cluster;            /* CTAs that share each inverse FFT (a thread-block cluster
                                over distributed shared memory): 1 when one CTA holds the
                                row (at most 16384 points), else 2 ... 16, each CTA holding
@@ -379,7 +382,7 @@ cwt_status cwt_execute(cwt_plan plan, const void *d_signal, void *d_complex, voi
  * device can address (cudaHostAlloc / cudaMallocHost, cudaHostRegister with
  * mapping, e.g. torch pin_memory(); 16-byte aligned) is written directly by
  * the kernels' epilogues over the host link, with no staging copy, unless the
- * outputs exceed 48 MB and the plan runs scales by residue classes: those are
+ * outputs exceed 6 MB and the plan runs scales by residue classes: those are
  * staged and copied in slices of channels while the next are computed.  Any
  * other output goes to a device staging buffer and is copied back.  Staging buffers
  * are allocated on the first call and kept by the plan.  Same layouts as
@@ -401,7 +404,7 @@ cwt_status cwt_execute_host(cwt_plan plan, const void *h_signal, void *h_complex
  *   d_complex / d_power / d_phase  device packed outputs (exactly the plan's kinds)
  * Requires an F32 plan.  The first batch of a new shape generates the banks
  * for its lengths and a workspace for the spectra's kept bins, up to 256 MB or
- * one epoch's (allocating and waiting); later batches of the same shape only
+ * one epoch's, less where memory is short (allocating and waiting); later batches of the same shape only
  * launch.  Asynchronous on `stream` otherwise.  Not inside a stream capture
  * (CWT_ECUDA).
  * CWT_EUNSUPPORTED for F64 plans, smooth-padded plans, or epochs whose
@@ -431,7 +434,9 @@ typedef struct {
     int max_streams;          /* stream slots (default 32) */
     int window;               /* W = N; only 2048 is built */
     double hop_seconds;       /* hop length in seconds (default 0.05) */
-    size_t mem_budget_bytes;  /* device bytes for streams (0 = no limit) */
+    size_t mem_budget_bytes;  /* bytes for banks and streams (0 = no limit): device
+                                 memory, and the results of batches in flight in the
+                                 page-locked host memory that the kernel writes */
     unsigned output_kinds;    /* only CWT_OUT_POWER is built */
     int reserved0;
     double gmw_gamma;         /* gamma for CWT_WAVELET_GMW (default 3) */
@@ -444,7 +449,7 @@ typedef struct {
     long long admitted, refused;  /* cwt_stream_open outcomes since the last reset */
     long long hops, launches;     /* hops completed, batched launches */
     long long coefficients;       /* power values delivered (C * S * H per hop) */
-    size_t device_bytes;          /* device memory held by banks and streams */
+    size_t device_bytes;          /* what counts against mem_budget_bytes */
     double latency_p50_s, latency_p99_s, latency_max_s, latency_mean_s;
     double span_s;                /* first hop ready -> last hop done */
 } cwt_server_stats_t;
@@ -461,7 +466,7 @@ cwt_status cwt_server_destroy(cwt_server srv);
 /* Admit a stream of `channels` channels sampled at fs Hz (every frequency must
  * be < fs/2 and representable on the window's W-point grid at fs, as in
  * cwt_plan_create; else CWT_EINVAL).  CWT_EBUSY when no slot is free or its
- * device memory would exceed the budget (the refusal is counted).  Generates
+ * memory would exceed the budget (mem_budget_bytes; the refusal is counted).  Generates
  * the bank for a new fs and grows the server's batch buffers to hold
  * kMaxPending (8) hops of every open stream, waiting for the batches in
  * flight if it has to replace them.  Call cwt_stream_open, cwt_server_step
@@ -577,12 +582,11 @@ cwt_status cwt_measure_peak(int what, double *tflops);
  * address and writes its twiddle table, then waits for that on `stream`.  No
  * call may be made inside a stream capture (CWT_ECUDA): a graph would replay
  * into the shared array at times that its caller does not order.
- * The address is kept for the
- * life of the process: do not call this entry point again on a device after
- * cudaDeviceReset.  Every call passes up to 128 scales on by value and
- * copies more from the host (so the caller may reuse them as soon as the call returns), reuses the same
- * array and overwrites everything it reads, so nothing needs clearing between
- * calls; calls that overlap on the GPU (unordered streams, other host
+ * The address is kept for the life of the process: do not call this entry point
+ * again on a device after cudaDeviceReset.  Every call passes up to 128 scales on
+ * by value and copies more from the host (so the caller may reuse the lists as
+ * soon as the call returns), reuses the same array and overwrites everything it
+ * reads, so nothing needs clearing between calls; calls that overlap on the GPU (unordered streams, other host
  * threads) race on it and must be serialised by the caller.  Its kernels run
  * on `stream`; the call returns without waiting for them (except the first
  * call's set-up).

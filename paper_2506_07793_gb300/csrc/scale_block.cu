@@ -217,4 +217,3 @@ cudaError_t launch_scale_block(const cwt_plan_s *p, void *out_c, void *out_p, vo
 }
 
 }  // namespace cwtk
-

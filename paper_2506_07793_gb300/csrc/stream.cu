@@ -343,8 +343,8 @@ cudaError_t grow_slots(cwt_server_s *srv, size_t items) {
     return cudaSuccess;
 }
 
-// What a stream counts against the server's budget: its ring and, in the
-// pinned queue that the kernel writes, the results of the batches in flight.
+// What a stream counts against the server's budget: its ring on the device and, in
+// the pinned queue that the kernel writes, the results of the batches in flight.
 size_t stream_dev_bytes(const cwt_server_s *srv, int C, int H) {
     const size_t ring = sizeof(float) * (size_t)C * (kSW + (size_t)kMaxPending * H);
     const size_t outs = sizeof(float) * (size_t)C * srv->S * H * kMaxPending * kSlots;
