@@ -203,7 +203,8 @@ double column_cost(int i, const ZoomShape &z) {
     else if (!z.both) f = eighth ? 0.95 : R >= 32 ? 1.0 : 1.1;
     else if (quarter) f = eighth ? 1.15 : 1.25;
     else if (P <= 8) f = three ? 1.35 : R >= 8 ? 1.95 : 1.35;
-    else f = P <= 16 ? 1.85 : R >= 128 ? 1.3 : R >= 64 ? 1.45 : 1.75;
+    else f = P <= 16 ? 1.85 : R >= 128 ? 1.3 : R >= 64 ? 1.45 : R > P ? 1.75 : 1.55;  // R <= P: a CTA holds the row
+    if (z.both && P > 4 && !quarter) f = 1.15 + (f - 1.15) * z.kept();
     if (R % P != 0 && P % R != 0) f *= 1.05;  // column groups that meet several rows form more band products
     // a division per output, and fewer of them stored
     if (z.sub != 1) f = three ? 1.25 : z.both ? 1.75 : 1.45;
@@ -234,7 +235,7 @@ double wide_cost(int i, int j, const ZoomShape &z) {
     const WideInst &w = wide_rest(j);
     const int Rp = z.M / (w.QB * w.QC), QA = wide_radix(i), R = Rp / QA;
     const bool eighth = Rp % 8 == 0 && z.n_out % 8 == 0, quarter = Rp % 4 == 0 && z.n_out % 4 == 0;
-    double f = z.both ? (eighth ? 1.15 : quarter ? 1.25 : 1.75) : eighth ? 0.95 : 1.0;
+    double f = z.both ? (eighth ? 1.15 : quarter ? 1.25 : 1.15 + 0.6 * z.kept()) : eighth ? 0.95 : 1.0;
     if (z.sub != 1) f = 1.6;
     const double pad = (double)((Rp + w.P - 1) / w.P * w.P) / Rp;
     const double first = (QA <= 8 ? 1.4 : 1.4 + 0.025 * (QA - 8) + (QA > 16 ? 0.02 * (QA - 16) : 0.0)) +

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "zoom.cuh"
@@ -68,6 +69,8 @@ struct ZoomShape {
     bool phase, both;
     bool rows_only, wide;  // only zoom_row_kernel; zoom_wide.cuh allowed
     double channels;  // nominal, for the cost of a launch against that of its rows
+    // the part of the row that the outputs cover
+    double kept() const { return n_out ? std::min(1.0, (double)n_out * sub / M) : 1.0; }
 };
 
 // Splits S scales with bands band[2 s] (start), band[2 s + 1] (length) into
